@@ -149,10 +149,15 @@ lgf_status lgf_plan_create(const int32_t *block_ijk, int64_t n_blocks, int32_t n
  *                      field of the separate form: the 4^3 source blocks of a
  *                      sibling group, fully unrolled)
  *   interval_kernel    product kernel of levels >= 1 (and of the merged
- *                      level-0/1 pass): 0 = default (5 for FP32 plans where a
- *                      level has >= 48 sibling groups; elsewhere one CTA per
- *                      (frequency chunk, group range) with the packed FP32
- *                      products of form 5, 8 warps), 1 = one frequency per
+ *                      level-0/1 pass): 0 = default (the merged pass by whole
+ *                      sibling groups: the 2 n_b cube of a group is transformed
+ *                      at once, padded to 4 n_b, and takes 27 products per
+ *                      frequency instead of 8 x 27; levels >= 1: 5 for FP32
+ *                      plans where a level has >= 48 sibling groups, elsewhere
+ *                      one CTA per (frequency chunk, group range) with the
+ *                      packed FP32 products of form 5, 8 warps).  Any other
+ *                      value keeps the blocks' own transforms of 2 n_b in the
+ *                      merged pass: 1 = one frequency per
  *                      thread, one CTA per (frequency chunk, group range), one
  *                      FMA per real product, 3 = two sibling groups per warp
  *                      sharing coefficient loads (2 is not a form: the two-
@@ -180,8 +185,8 @@ lgf_status lgf_plan_create(const int32_t *block_ijk, int64_t n_blocks, int32_t n
  *                      the parent neighbourhood (343 kernel offsets) and one
  *                      inverse FFT.  1: separate level-1 transforms of length
  *                      S_I, as the level interactions of Sec. 3.1 are listed.
- *   free_sms           schedule of the persistent products (interval_kernel
- *                      form 4): -1 = they take every SM and levels >= 2 run
+ *   free_sms           schedule of the persistent level-0 products (interval_kernel
+ *                      4 and 5; no effect on the grouped form): -1 = they take every SM and levels >= 2 run
  *                      before and after them; k > 0 = they take all but k SMs
  *                      and levels >= 2 run beside them on the rest; 0 = the
  *                      library's choice
@@ -192,8 +197,8 @@ lgf_status lgf_plan_create(const int32_t *block_ijk, int64_t n_blocks, int32_t n
  *                      memory, each block's input, spectrum and output moved
  *                      by bulk copies that overlap the neighbouring blocks'
  *                      passes, each line transform split into output classes
- *                      (FP32 plans with n_b 8 or 16); 0 = 1 (the faster form
- *                      as measured)
+ *                      (FP32 plans with n_b 8 or 16; it transforms the blocks,
+ *                      so the merged pass keeps their own spectra); 0 = 1
  *   level_order        per-level interpolation orders (Sec. 4 notes that the
  *                      interval sizes and stencils may be tuned per level):
  *                      level_order[k] is the polynomial degree of the stencil
@@ -216,8 +221,8 @@ lgf_status lgf_plan_create(const int32_t *block_ijk, int64_t n_blocks, int32_t n
  *                      neighbour groups) a CTA takes for one frequency chunk,
  *                      rounded up to whole warps; 0 = chosen from the level's
  *                      size (about four waves of CTAs)
- * All variants compute the same sums (Eq. alg_mult); they differ only in
- * scheduling.
+ * All variants compute the same sums (Eq. alg_mult); they differ in scheduling
+ * and in the transforms that the sums run on.
  */
 #define LGF_LEVEL_ORDERS 8
 typedef struct {
@@ -264,7 +269,9 @@ lgf_status lgf_plan_create_multi(const int32_t *block_ijk, const int64_t *block_
  *   pairs[l]   level 0: near (block, block) pairs; level l >= 1: interaction-list
  *              (target, source) interval pairs; each costs NW complex products
  *   intervals[l], groups[l]   intervals and sibling groups per level
- *   nw[l]      frequencies per spectrum at level l (0 where l has no products)
+ *   nw[l]      frequencies per spectrum at level l (0 where l has no products);
+ *              levels 0 and 1: of a block's own spectrum (length 2 n_b), also
+ *              where the merged pass runs by whole sibling groups
  *   top_product_level  highest level with a non-empty interaction list
  *   merged_level01     1 if levels 0 and 1 share one product pass (nw[1] is
  *                      then the level-0 spectrum size)
@@ -423,7 +430,8 @@ lgf_status lgf_plan_timings(lgf_plan plan, int32_t max_kernels, int32_t *n_kerne
  * kernel launch.  A CTA takes a block through the forward transform, the
  * product with the block's own kernel spectrum and the inverse transform with
  * the spectrum in shared memory (it never reaches device memory); the results
- * equal those of a one-block plan and of lgf_solve_blocks_noalloc.
+ * equal those of lgf_solve_blocks_noalloc, and to rounding those of a
+ * one-block plan.
  *
  *   f_dev, u_dev  device pointers, n_blocks * n_b^3 values of the precision,
  *                 block-major with x fastest (as lgf_solve); f_dev == u_dev

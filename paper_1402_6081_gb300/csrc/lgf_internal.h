@@ -27,7 +27,7 @@ std::shared_ptr<const std::vector<double>> green_abs_table(int h, int V);
 // In-place complex DFT of length n with sign -1 (forward) or +1 (inverse,
 // unnormalised), on a strided sequence.
 void fft_inplace(std::complex<double>* x, int n, int stride, int sign);
-// count lines at base + c*line_stride, each n elements at stride (n <= 96).
+// count lines at base + c*line_stride, each n elements at stride (n <= 128).
 void fft_lines(std::complex<double>* base, int n, int stride, int count, int64_t line_stride,
                int sign);
 

@@ -19,6 +19,7 @@
 #include <unordered_map>
 #include <unordered_set>
 
+#include "group.h"
 #include "lgf_internal.h"
 
 namespace lgf {
@@ -217,15 +218,17 @@ static std::map<SpecKey, std::weak_ptr<SpecEntry>> g_spec_cache;
 
 // kind: kNear (27 offsets |d| <= 1, n = n_b), kInterval (343 offsets |d| <= 3,
 // n = n_I, zero at the near ones), kBlock (343 offsets |d| <= 3, n = n_b, all
-// filled: level 0 near field and level-1 interaction list on the block grid)
-enum SpecKind { kNear = 0, kInterval = 1, kBlock = 2 };
+// filled: level 0 near field and level-1 interaction list on the block grid),
+// kGroup (the 27 offsets |d| <= 1 of sibling groups, cubes of 2 n_b points:
+// group.h)
+enum SpecKind { kNear = 0, kInterval = 1, kBlock = 2, kGroup = 3 };
 
 // oct (343-offset kinds only): store the 40 representatives of the offsets
 // under the reflections of G instead of the 172-row half table (the products
 // kernel maps each offset's frequencies onto its representative's)
 static lgf_status get_spectra(int device, int n_b, int S, int h, int kind, int prec,
                               std::shared_ptr<SpecEntry>& out, int oct = 0) {
-    if (kind == kNear) oct = 0;
+    if (kind == kNear || kind == kGroup) oct = 0;
     const SpecKey key{device, n_b, S, h, kind, prec, oct};
     std::lock_guard<std::mutex> lock(g_spec_mu);
     auto it = g_spec_cache.find(key);
@@ -235,18 +238,22 @@ static lgf_status get_spectra(int device, int n_b, int S, int h, int kind, int p
             return ok();
         }
     }
-    const bool near = kind == kNear;
-    const int n = kind == kInterval ? n_b + 1 : n_b;
-    const int V = near ? 2 * n_b - 1 : kind == kBlock ? 4 * n_b - 1 : 4 * n_b;
+    const bool near = kind == kNear, group = kind == kGroup;
+    // edge of the cubes that interact and the pitch of their offsets
+    const int n = group ? 2 * n_b : kind == kInterval ? n_b + 1 : n_b, pitch = group ? 2 * n_b : n_b;
+    const int V = near ? 2 * n_b - 1 : kind == kBlock || group ? 4 * n_b - 1 : 4 * n_b;
     auto tab = green_abs_table(h, V);
     // The kernel vector of -d is that of d reflected (G is even and the
     // window |m_a| <= n - 1 symmetric), so its spectrum is the complex
     // conjugate: the 343-offset tables keep only the rows id >= 171 (d = 0 and
     // the offsets after it in x-fastest order); row id < 171 is the conjugate
-    // of row 342 - id.  The 27-offset table is kept whole.
-    const int nd = near ? 27 : oct ? 40 : 172;
-    const int first = near ? 0 : 171;
-    const int64_t NW = nw_of(S), NWS = nws_of(S);
+    // of row 342 - id.  The groups' 27-offset table likewise keeps the rows id
+    // >= 13.  The near table is kept whole.
+    const int nd = near ? 27 : group ? kGroupRows : oct ? 40 : 172;
+    const int first = near ? 0 : group ? 27 - kGroupRows : 171;
+    const GroupShape gs = group ? group_shape(n_b) : GroupShape{};
+    const int64_t NW = nw_of(S);
+    const int64_t NWS = !group ? nws_of(S) : prec == LGF_FP64 ? NW : NW / S * 16 * gs.pairs;
     std::vector<std::complex<double>> all(size_t(nd) * NWS, 0.0);
     // offset of a stored row: the 27- or 343-offset id, or the representative
     // (|dx|, a, b), a <= b, of the reduced table (row 10 |dx| + b (b + 1) / 2 + a)
@@ -258,7 +265,7 @@ static lgf_status get_spectra(int device, int n_b, int S, int h, int kind, int p
             d[2] = b;
             return;
         }
-        const int id = first + row, r = near ? 3 : 7, o = near ? 1 : 3;
+        const int id = first + row, r = near || group ? 3 : 7, o = near || group ? 1 : 3;
         d[0] = id % r - o;
         d[1] = (id / r) % r - o;
         d[2] = id / (r * r) - o;
@@ -278,7 +285,30 @@ static lgf_status get_spectra(int device, int n_b, int S, int h, int kind, int p
                 const int row = todo[t];
                 int d[3];
                 offset_of(row, d);
-                kernel_spectrum(n_b, n, h, S, d, tab->data(), V, &all[size_t(row) * NWS]);
+                std::complex<double>* out_row = &all[size_t(row) * NWS];
+                if (!group) {
+                    kernel_spectrum(pitch, n, h, S, d, tab->data(), V, out_row);
+                    continue;
+                }
+                std::vector<std::complex<double>> w(static_cast<size_t>(NW));
+                kernel_spectrum(pitch, n, h, S, d, tab->data(), V, w.data());
+                const int64_t cols = NW / S;
+                for (int64_t c = 0; c < cols; ++c) {
+                    if (prec == LGF_FP64) {   // column by column, kz fastest
+                        for (int kz = 0; kz < S; ++kz) out_row[c * S + kz] = w[size_t(kz * cols + c)];
+                        continue;
+                    }
+                    // column by column, then row by row: kz = r + 8 m by r, the m in pairs
+                    // (re, re, im, im), the last half of an odd count zero
+                    std::complex<double>* o = &all[size_t((c * kGroupRows + row) * (16 * gs.pairs))];
+                    for (int r = 0; r < 8; ++r)
+                        for (int j = 0; j < gs.pairs; ++j, o += 2) {
+                            const std::complex<double> a = w[size_t((r + 16 * j) * cols + c)],
+                                                       b = 2 * j + 1 < gs.rb ? w[size_t((r + 16 * j + 8) * cols + c)] : 0.0;
+                            o[0] = {a.real(), b.real()};
+                            o[1] = {a.imag(), b.imag()};
+                        }
+                }
             }
         });
     for (auto& t : th) t.join();
@@ -286,7 +316,6 @@ static lgf_status get_spectra(int device, int n_b, int S, int h, int kind, int p
     e->device = device;
     const size_t elem = prec == LGF_FP64 ? sizeof(double) : sizeof(float);
     e->bytes = size_t(nd) * NWS * 2 * elem;
-    (void)NW;
     cudaError_t ce = cudaMalloc(&e->ptr, e->bytes);
     if (ce != cudaSuccess) {
         e->ptr = nullptr;
@@ -303,7 +332,7 @@ static lgf_status get_spectra(int device, int n_b, int S, int h, int kind, int p
         ce = cudaMemcpy(e->ptr, f.data(), e->bytes, cudaMemcpyHostToDevice);
     }
     if (ce != cudaSuccess) return cuda_fail(ce, "spectra upload");
-    e->has_tmap = !near && !oct && encode_table_map(*e, nd, NWS, prec);
+    e->has_tmap = !near && !group && !oct && encode_table_map(*e, nd, NWS, prec);
     g_spec_cache[key] = e;
     out = e;
     return ok();
@@ -417,6 +446,9 @@ struct lgf_plan_s {
     // first n_b nodes of a level-1 interval: their products are summed into
     // one spectrum per block (one inverse FFT, no level-1 transforms)
     bool merged = true;
+    // merged levels 0 and 1 by whole sibling groups (group.h)
+    bool grouped = false;
+    lgf::GroupTables grp;
     std::vector<lgf::DevLevel> lev;
     std::vector<int64_t> pairs, intervals, groups;   // per level, for lgf_plan_get_stats
     void* W = nullptr;                  // device copy (unused by the kernels, kept for tools)
@@ -568,6 +600,7 @@ struct HostLevel {
     int n_groups = 0;
     bool m2l = false;                          // interaction list not empty (level 0: near field, always)
     std::vector<int> gn;                       // n_groups x 27 neighbour groups, -1 = none
+    std::vector<I3> gpos;                      // level 0: the groups' indices
     std::vector<R2CItem> r2c;                  // src: block (l <= 1) or slot (l >= 2); dst: slot
     std::vector<int> iv_slot;                  // slot of each interval
     std::vector<int> reg_child, reg_parent;    // l >= 2: 8 children per parent (block at l = 2, else slot)
@@ -607,7 +640,7 @@ static bool uses_persist(const lgf_plan_s* P, int l) {
     if (P->prec != LGF_FP32) return false;
     if (!persist_supported(l == 0 ? P->S0 : P->SI)) return false;
     if (P->interval_kernel != 0 && P->interval_kernel != 4 && P->interval_kernel != 5) return false;
-    if (l == 0 && !P->merged) return false;
+    if (l == 0 && (!P->merged || P->grouped)) return false;
     // beside shared-SM level-0 products, levels >= 2 keep the
     // one-CTA-per-chunk form, which fits on the SMs left to them
     if (l >= 2 && shares_sms(P)) return false;
@@ -807,6 +840,7 @@ static lgf_status build_host(const int32_t* ijk, int64_t NB, int L, HostPlan& H)
         T.n_groups = int(L_.groups.size());
         T.m2l = l == 0 || m2l[size_t(l)];
         T.gn.assign(size_t(T.n_groups) * 27, -1);
+        if (l == 0) T.gpos = L_.groups;
         for (int g = 0; g < T.n_groups; ++g)
             for (int e = 0; e < 27; ++e) {
                 const I3& G = L_.groups[size_t(g)];
@@ -841,6 +875,95 @@ static lgf_status build_host(const int32_t* ijk, int64_t NB, int L, HostPlan& H)
         }
     }
     return ok();
+}
+
+// Tables and buffers of the grouped level-0/1 convolution: the children's
+// blocks and level-1 slots of every group, and the sets of 2^3 target groups
+// with the 4^3 groups around them (n_groups1: groups at level 1).  A set never spans two problems, and its
+// place depends on the group indices alone, so a problem's sums run in the
+// same order whatever other problems share the plan.
+static lgf_status build_group(lgf_plan_s* P, const std::vector<HostPlan>& hp, const std::vector<int>& boff,
+                              const std::vector<std::vector<int>>& goff, int n_groups1, DevLevel& D, size_t cplx) {
+    std::vector<int> blk(size_t(D.n_groups) * 8, -1), aux(size_t(D.n_groups) * 8, -1), sup;
+    for (size_t p = 0; p < hp.size(); ++p) {
+        const HostPlan& H = hp[p];
+        const HostLevel& T = H.lev[0];
+        const int g0 = goff[0][p];
+        for (int64_t b = 0; b < H.n_blocks; ++b) {
+            const int s = T.iv_slot[size_t(b)];
+            blk[size_t(s) + 8 * size_t(g0)] = int(b) + boff[p];
+            // the same slot number at level 1, whose group list is level 0's
+            if (H.Lmac >= 2) aux[size_t(s) + 8 * size_t(g0)] = s + 8 * goff[1][p];
+        }
+        std::unordered_map<uint64_t, int> at;
+        for (size_t g = 0; g < T.gpos.size(); ++g) at[pack(T.gpos[g])] = int(g) + g0;
+        // groups are in Morton order, so the sets come so too
+        std::unordered_set<uint64_t> seen;
+        for (const I3& g : T.gpos) {
+            const I3 q = parent_of(g);
+            if (!seen.insert(pack(q)).second) continue;
+            auto id = [&](int x, int y, int z) {
+                const auto it = at.find(pack({2 * q[0] + x, 2 * q[1] + y, 2 * q[2] + z}));
+                return it == at.end() ? -1 : it->second;
+            };
+            for (int i = 0; i < 64; ++i) sup.push_back(id(i % 4 - 1, (i / 4) % 4 - 1, i / 16 - 1));
+            for (int c = 0; c < 8; ++c) sup.push_back(id(c & 1, (c >> 1) & 1, c >> 2));
+        }
+    }
+    lgf_status s;
+    if ((s = check_range("group block", blk, -1, P->n_blocks)) != LGF_OK) return s;
+    if ((s = check_range("group level-1 slot", aux, -1, 8LL * n_groups1)) != LGF_OK) return s;
+    if ((s = check_range("group set", sup, -1, D.n_groups)) != LGF_OK) return s;
+    const int S = 4 * P->n_b;
+    const size_t column_set = size_t(D.n_groups) * size_t(group_columns(P->n_b)) * cplx;
+    const bool f32 = P->prec == LGF_FP32;
+    if ((s = dalloc(P, column_set * size_t(f32 ? S / 2 : S), &D.fh, false)) != LGF_OK) return s;
+    if ((s = dalloc(P, column_set * size_t(S / 2), &D.uh, false)) != LGF_OK) return s;
+    int *dblk = nullptr, *daux = nullptr, *dsets = nullptr;
+    if ((s = upload(P, blk, &dblk)) != LGF_OK) return s;
+    if ((s = upload(P, aux, &daux)) != LGF_OK) return s;
+    std::vector<int> sets;
+    sets.reserve(sup.size() / 72 * kSetInts);
+    for (size_t i = 0; i < sup.size(); i += 72) {
+        int rows = 0;
+        for (size_t k = 0; k < 64; ++k) {
+            if (sup[i + k] >= 0) rows |= 1 << (k / 4);
+            sets.push_back(sup[i + k] >= 0 || !f32 ? sup[i + k] : D.n_groups);
+        }
+        sets.insert(sets.end(), sup.begin() + long(i) + 64, sup.begin() + long(i) + 72);
+        sets.insert(sets.end(), {rows, 0, 0, 0});
+    }
+    if ((s = upload(P, sets, &dsets)) != LGF_OK) return s;
+    P->grp.n_groups = D.n_groups;
+    P->grp.n_super = int(sup.size() / 72);
+    P->grp.blk = dblk;
+    P->grp.aux = daux;
+    P->grp.sets = reinterpret_cast<const int4*>(dsets);
+    if (f32) {
+        // bands of whole column sets whose images fill about 48 MB of L2
+        const GroupShape gs = group_shape(P->n_b);
+        const int64_t column = int64_t(D.n_groups + 1) * gs.image * int64_t(cplx);
+        const int64_t nc = group_columns(P->n_b), most = std::max<int64_t>(32, int64_t(48 << 20) / column);
+        const int64_t bands = (nc + most - 1) / most;
+        P->grp.band_cols = int(std::min((nc / bands + 31) / 32 * 32, nc));
+        if ((s = dalloc(P, size_t(column) * size_t(P->grp.band_cols), &P->grp.images, true)) != LGF_OK) return s;
+    }
+    std::vector<double> t(2 * size_t(S));
+    for (int m = 0; m < S; ++m) {
+        const double a = 2.0 * M_PI * double(m) / double(S);
+        t[2 * size_t(m)] = std::cos(a);
+        t[2 * size_t(m) + 1] = std::sin(a);
+    }
+    if (P->prec == LGF_FP64) {
+        double* d = nullptr;
+        if ((s = upload(P, t, &d)) != LGF_OK) return s;
+        P->grp.tw = d;
+    } else {
+        float* d = nullptr;
+        if ((s = upload(P, std::vector<float>(t.begin(), t.end()), &d)) != LGF_OK) return s;
+        P->grp.tw = d;
+    }
+    return get_spectra(P->device, P->n_b, S, 1, kGroup, P->prec, D.kh);
 }
 
 // Concatenates the problems' tables level by level and builds the device
@@ -922,7 +1045,9 @@ static lgf_status build_plan(lgf_plan_s* P, const std::vector<HostPlan>& hp) {
         D.m2l = (l == 0) || (any && !(l == 1 && P->merged));
         const size_t slots = size_t(D.n_groups) * 8;
         lgf_status s;
-        if (D.m2l) {
+        if (l == 0 && P->grouped) {
+            if ((s = build_group(P, hp, boff, goff, Lmac >= 1 ? ngroups[1] : 0, D, cplx)) != LGF_OK) return s;
+        } else if (D.m2l) {
             const int S = l == 0 ? P->S0 : P->SI;
             const size_t NWS = size_t(nws_of(S));
             if ((s = dalloc(P, slots * NWS * cplx, &D.fh, true)) != LGF_OK) return s;
@@ -1032,7 +1157,7 @@ static lgf_status build_plan(lgf_plan_s* P, const std::vector<HostPlan>& hp) {
     }
     // level-0 output items: block b from its level-0 slot, plus its level-1
     // field (same slot number within the problem, level-1 group offset)
-    {
+    if (!P->grouped) {
         std::vector<C2RItem> items;
         for (size_t p = 0; p < np; ++p) {
             const HostPlan& H = hp[p];
@@ -1114,6 +1239,7 @@ static lgf_status build_plan(lgf_plan_s* P, const std::vector<HostPlan>& hp) {
         for (int l = 0; l <= Lmac; ++l) {
             DevLevel& D = P->lev[size_t(l)];
             const int S = l == 0 ? P->S0 : P->SI;
+            if (l == 0 && P->grouped) continue;
             if (P->prec == LGF_FP32 && fft_large_supported(S, nb) && (l == 0 || fft_large_supported(S, nI)))
                 continue;
             const size_t items = size_t(std::max({D.n_r2c, D.n_c2r, l == 0 ? P->n_out : 0}));
@@ -1219,6 +1345,7 @@ static lgf_status solve_impl(lgf_plan_s* P, const T* f, T* u, cudaStream_t st) {
     auto wait = [&](cudaStream_t s, int k) { return conc ? cudaStreamWaitEvent(s, P->join[k], 0) : cudaSuccess; };
     // level-0 inverse FFT into u, plus the level-1 field add when given
     auto c2r0 = [&](const T* add) -> cudaError_t {
+        if (P->grouped) return Group<T>::inverse(nb, P->grp, group_banded<T>() ? lev[0].fh : lev[0].uh, u, add, nI, n3, st);
         if constexpr (std::is_same_v<T, float>)
             if (P->fft_kernel == 2)
                 return c2r_cube(P->S0, nb, lev[0].uh, P->out_items, P->n_out, u, b3, add, nI, n3, P->cube_grid[1],
@@ -1333,6 +1460,7 @@ static lgf_status solve_impl(lgf_plan_s* P, const T* f, T* u, cudaStream_t st) {
     }
     // ---- level 0 on the caller's stream: forward FFT, near-field products
     e = timed(P, "r2c_level0", st, [&] {
+        if (P->grouped) return Group<T>::forward(nb, P->grp, f, lev[0].uh, lev[0].fh, st);
         if constexpr (std::is_same_v<T, float>)
             if (P->fft_kernel == 2) {
                 if (P->in_map_src != f)
@@ -1347,6 +1475,9 @@ static lgf_status solve_impl(lgf_plan_s* P, const T* f, T* u, cudaStream_t st) {
     if (split) LGF_CUDA(wait(st, 1));
     if (P->merged) {
         e = timed(P, "mac_level01", st, [&] {
+            if (P->grouped)
+                return Group<T>::products(nb, P->grp, group_banded<T>() ? lev[0].uh : lev[0].fh, lev[0].kh->ptr,
+                                          group_banded<T>() ? lev[0].fh : lev[0].uh, st);
             // directly behind the forward FFT on st (no event between them):
             // launched early, it stages its first coefficient chunks meanwhile
             const int early = !split && P->ev.empty() ? 1 : 0;
@@ -1558,6 +1689,9 @@ static lgf_status create_plan(const int32_t* block_ijk, const int64_t* offsets, 
             P->nmax_lv[size_t(k) + 2] = o + 1;
         }
     }
+    // The grouped form unless the options ask for a product or transform form
+    // of the blocks' own spectra.
+    P->grouped = P->merged && P->interval_kernel == 0 && P->fft_kernel != 2 && group_supported(n_b);
     lgf_status s = ensure_twiddles(P->device, precision);
     if (s != LGF_OK) return s;
     std::vector<HostPlan> hp(static_cast<size_t>(n_problems));
@@ -1610,7 +1744,7 @@ static lgf_status create_plan(const int32_t* block_ijk, const int64_t* offsets, 
     LGF_CUDA(cudaDeviceGetStreamPriorityRange(&prio_low, &prio_high));
     LGF_CUDA(cudaStreamCreateWithFlags(&P->aux[0], cudaStreamNonBlocking));
     const bool split = P->free_sms < 0 && uses_persist(P.get(), 0);
-    LGF_CUDA(cudaStreamCreateWithPriority(&P->aux[1], cudaStreamNonBlocking, split ? prio_high : prio_low));
+    LGF_CUDA(cudaStreamCreateWithPriority(&P->aux[1], cudaStreamNonBlocking, split || P->grouped ? prio_high : prio_low));
     LGF_CUDA(cudaEventCreateWithFlags(&P->fork, cudaEventDisableTiming));
     for (auto& j : P->join) LGF_CUDA(cudaEventCreateWithFlags(&j, cudaEventDisableTiming));
     *out = P.release();
