@@ -18,7 +18,7 @@
 
 namespace lgf {
 
-// Columns (kx, ky) of a group's spectrum; a column is one z line.
+// Columns kx S + ky of a group's spectrum; a column is one z line.
 inline int64_t group_columns(int n_b) { return int64_t(4 * n_b) * (2 * n_b + 1); }
 // Stored rows of the kernel table: offsets id 13 .. 26 of 27 (x fastest), row
 // id - 13; offset 26 - id is the conjugate.  A row holds column (ky * NX + kx)

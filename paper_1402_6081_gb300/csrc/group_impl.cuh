@@ -15,10 +15,12 @@
 // stage reads both spectra from the pair as it loads, so separating them
 // costs no pass.
 //
-// Layouts: xy[ky * NX + kx][group][z], spec[ky * NX + kx][group][kz]: a z line
-// is contiguous, and a column's lines of consecutive groups (Morton order, so
-// mostly neighbours) follow one another, which makes the sources of a tile a
-// few long runs; a plane's values are written PZ planes (32 bytes) at a time.
+// Layouts.  A column is kx * S + ky.  xy[group][z / PZ][column][z % PZ]: what a
+// plane kernel's CTA writes or reads is contiguous, whole cache lines per warp
+// access (with a line's z values side by side it moved 32 bytes per request,
+// and the requests in flight, not the bytes, bounded it: 128^3 inverse 37 us);
+// a z kernel takes tens of consecutive columns of a group.  Spectra are
+// [column][group][..]: the sources of a set lie near one another.
 #pragma once
 
 #include <algorithm>
@@ -37,23 +39,26 @@ struct Dim {
     static constexpr int N = 2 * NB, S = 4 * NB, NX = S / 2 + 1, RB = NB / 2;
     static constexpr int LP = RB | 1;                  // pitch of an 8 x RB exchange: odd
     static constexpr int64_t NC = int64_t(S) * NX;     // columns
-    // plane kernels: PZ planes per CTA, each with NB row pairs of S values
-    // (ZB) and an exchange (EB) that serves the x and the y passes
+    // Plane kernels: PZ planes per CTA of 8 warps (16 for the long lines, whose
+    // shared memory leaves room for one CTA per SM).  A team of 8 lanes per
+    // plane takes LN lines through both stages, exchanging them in the warp's
+    // own buffer (XB values).
+    static constexpr int TH = RB <= 8 ? 256 : 512;
+    static constexpr int LN = RB <= 8 ? 8 / RB : 1, R1 = (LN * RB + 7) / 8, R2 = LN;
+    static constexpr int TEAMS(int pz) { return 4 / pz; }   // teams of a warp for the same plane
+    static constexpr int XB(int pz) { return TEAMS(pz) * LN * 8 * RB * pz; }
     static constexpr size_t smem(int pz) {
-        return sizeof(cx<T>) * (size_t(NB) * S * pz + exch(pz) + S);
+        return sizeof(cx<T>) * (size_t(4 * RB) * NX * pz + size_t(TH / 32) * XB(pz) + S);
     }
-    // distance of two planes in the x exchange: 4 mod 16 complex values, so
-    // four planes times four consecutive c or b fall into different banks
-    static constexpr int xplane() { return ((NB * 8 * LP + 11) / 16) * 16 + 4; }
-    static constexpr size_t exch(int pz) {
-        const size_t x = size_t(xplane()) * pz, y = size_t(S) * NX * pz;
-        return x > y ? x : y;
-    }
-    static constexpr int pick() { return smem(4) <= 220 * 1024 ? 4 : smem(2) <= 220 * 1024 ? 2 : 1; }
-    static constexpr int PZ = pick();
-    static constexpr int threads() {
-        const int tasks = 8 * NX * PZ, rounds = (tasks + 383) / 384;
-        return ((tasks + rounds - 1) / rounds + 31) / 32 * 32;
+    static constexpr int PZ = smem(4) <= 200 * 1024 ? 4 : smem(2) <= 200 * 1024 ? 2 : 1;
+    // xy index of z 0 of a column of a group; z adds zoff(z)
+    __host__ __device__ static constexpr int64_t xy(int g, int col) { return (int64_t(g) * (N / PZ) * NC + col) * PZ; }
+    __host__ __device__ static constexpr int64_t zoff(int z) { return int64_t(z / PZ) * NC * PZ + z % PZ; }
+    // a line's value (c, b) in the exchange buffer: the low bits of b exchanged
+    // by c where RB is a power of two, so that both stages' accesses (four
+    // planes times four consecutive b or c) fall into different banks
+    __host__ __device__ static constexpr int at(int c, int b) {
+        return c * RB + (RB == 2 ? b ^ ((c >> 1) & 1) : (RB & (RB - 1)) == 0 ? b ^ (c & 3) : b);
     }
     // products: whole columns per CTA, about 128 frequencies
     static constexpr int COLS = S >= 128 ? 1 : 128 / S;
@@ -82,118 +87,171 @@ __device__ __forceinline__ cx<T> ld(const cx<T>* p) {
 }
 
 // ---------------------------------------------------------------------------
+// Plane kernels.  Between the x and the y pass the PZ planes are in shared
+// memory as Z[q RB + b][kx][plane]: the complex line of the rows y = l and
+// l + n_b (l = b for q < 2, b + RB above) at kx (q even) or S - kx (q odd), so
+// the y pass of one kx reads column kx of it alone and both passes exchange
+// their stages within a warp; the one CTA barrier is between the passes.  Bound
+// by latency at 128^3 (17 us forward, 22 us inverse; bytes alone 6.4), near the
+// memory in large domains: 512^3 tori, forward 1.37 GB in 0.28 ms, inverse with
+// the level-1 field 1.75 GB in 0.40 ms (5 TB/s).
+template <typename T, int NB>
+struct Plane {
+    using D = Dim<T, NB>;
+    static constexpr int RB = D::RB, S = D::S, NX = D::NX, PZ = D::PZ, TEAMS = D::TEAMS(PZ);
+    static constexpr int LINES = TEAMS * D::LN;   // lines of a warp's step
+    cx<T>* Z;
+    cx<T>* X;          // this warp's exchange buffer
+    const cx<T>* tw;
+    int pz, team, lane8;
+    __device__ __forceinline__ Plane(unsigned char* smem, const cx<T>* tw_dev) {
+        Z = reinterpret_cast<cx<T>*>(smem);
+        cx<T>* tws = Z + 4 * RB * NX * PZ;
+        const int lane = int(threadIdx.x % 32);
+        X = tws + S + int(threadIdx.x / 32) * D::XB(PZ);
+        tw = tws;
+        pz = lane % PZ;
+        lane8 = (lane / PZ) % 8;
+        team = lane / (PZ * 8);
+        for (int i = threadIdx.x; i < S; i += D::TH) tws[i] = ld(tw_dev + i);
+    }
+    // round r of a stage of PER tasks per line: line within the step, task
+    template <int PER>
+    __device__ __forceinline__ bool task(int r, int& line, int& pos) const {
+        const int i = r * 8 + lane8;
+        line = team * D::LN + i / PER;
+        pos = i % PER;
+        return i < D::LN * PER;
+    }
+    __device__ __forceinline__ cx<T>& x(int line, int c, int b) { return X[(line * 8 * RB + D::at(c, b)) * PZ + pz]; }
+    __device__ __forceinline__ cx<T>& z(int q, int b, int kx) { return Z[((q * RB + b) * NX + kx) * PZ + pz]; }
+    // Z of the complex line l at frequency k
+    __device__ __forceinline__ cx<T> line_at(int l, int k) {
+        const int q = l < RB ? 0 : 2, b = l < RB ? l : l - RB;
+        return 2 * k <= S ? z(q, b, k) : z(q + 1, b, S - k);
+    }
+    __device__ __forceinline__ void put_line(int l, int k, cx<T> v) {
+        const int q = l < RB ? 0 : 2, b = l < RB ? l : l - RB;
+        if (2 * k <= S) z(q, b, k) = v;
+        if (2 * k >= S || k == 0) z(q + 1, b, k == 0 ? 0 : S - k) = v;
+    }
+};
+
 // Forward x and y transforms of PZ planes of a group.
 template <typename T, int NB>
-__global__ void __launch_bounds__(Dim<T, NB>::threads()) k_gxy_fwd(const T* __restrict__ f, const int* __restrict__ blk,
-                                                                   const cx<T>* __restrict__ tw, cx<T>* __restrict__ xy,
-                                                                   int n_groups) {
+__global__ void __launch_bounds__(Dim<T, NB>::TH, sizeof(T) == 4 && NB <= 16 ? 4 : 1)
+    k_gxy_fwd(const T* __restrict__ f, const int* __restrict__ blk, const cx<T>* __restrict__ tw,
+              cx<T>* __restrict__ xy) {
     using D = Dim<T, NB>;
-    constexpr int N = D::N, S = D::S, NX = D::NX, RB = D::RB, LP = D::LP, PZ = D::PZ, TH = D::threads();
+    using P = Plane<T, NB>;
+    constexpr int N = D::N, S = D::S, NX = D::NX, RB = D::RB, PZ = D::PZ, WARPS = D::TH / 32;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    cx<T>* ZB = reinterpret_cast<cx<T>*>(smem_raw);      // [NB pairs][S][PZ]
-    cx<T>* EB = ZB + NB * S * PZ;
-    cx<T>* tws = EB + D::exch(PZ);
-    const int g = blockIdx.x / (N / PZ), z0 = (blockIdx.x % (N / PZ)) * PZ;
-    const int* gb = blk + int64_t(g) * 8;
-    for (int i = threadIdx.x; i < S; i += TH) tws[i] = ld(tw + i);
-    __syncthreads();
-    // x stage 1: the thread of (plane, b, pair l); rows y = l and l + n_b
-    for (int t = threadIdx.x; t < PZ * RB * NB; t += TH) {
-        const int pz = t % PZ, b = (t / PZ) % RB, l = t / (PZ * RB);
-        const int z = z0 + pz, cz = z >= NB ? 4 : 0;
-        const int64_t row = int64_t(z - (cz ? NB : 0)) * NB * NB + l * NB;
-        cx<T> x[8];
+    P p(smem_raw, tw);
+    const int g = blockIdx.x / (N / PZ), z = int(blockIdx.x % (N / PZ)) * PZ + p.pz, cz = z >= NB ? 4 : 0;
+    const int warp = int(threadIdx.x / 32);
+    // the plane's four blocks: x half, then y half
+    int blocks[4];
 #pragma unroll
-        for (int a = 0; a < 4; ++a) {
-            const int cxx = a >> 1;   // RB a + b < n_b for a < 2
-            const int b0 = __ldg(gb + cxx + cz), b1 = __ldg(gb + cxx + 2 + cz);
-            const int64_t at = row + (RB * a + b - (cxx ? NB : 0));
-            x[a].x = b0 >= 0 ? __ldg(f + int64_t(b0) * (NB * NB * NB) + at) : T(0);
-            x[a].y = b1 >= 0 ? __ldg(f + int64_t(b1) * (NB * NB * NB) + at) : T(0);
+    for (int i = 0; i < 4; ++i) blocks[i] = __ldg(blk + int64_t(g) * 8 + i + cz);
+    const int64_t zrow = int64_t(z - (cz ? NB : 0)) * NB * NB;
+    __syncthreads();
+    for (int l0 = warp * P::LINES; l0 < NB; l0 += WARPS * P::LINES) {
+#pragma unroll
+        for (int r = 0; r < D::R1; ++r) {
+            int line, b;
+            if (!p.template task<RB>(r, line, b) || l0 + line >= NB) continue;
+            cx<T> x[8];
+#pragma unroll
+            for (int a = 0; a < 4; ++a) {   // RB a + b < n_b for a < 2
+                const int64_t at = zrow + (l0 + line) * NB + (RB * (a & 1) + b);
+                const int b0 = blocks[a >> 1], b1 = blocks[(a >> 1) + 2];
+                x[a].x = b0 >= 0 ? __ldg(f + int64_t(b0) * (NB * NB * NB) + at) : T(0);
+                x[a].y = b1 >= 0 ? __ldg(f + int64_t(b1) * (NB * NB * NB) + at) : T(0);
+            }
+#pragma unroll
+            for (int a = 4; a < 8; ++a) x[a] = czero<T>();
+            dft<8, -1, 4>(x);
+#pragma unroll
+            for (int c = 0; c < 8; ++c) p.x(line, c, b) = cmulc(x[c], p.tw[b * c]);
         }
+        __syncwarp();
 #pragma unroll
-        for (int a = 4; a < 8; ++a) x[a] = czero<T>();
-        dft<8, -1, 4>(x);
-        cx<T>* e = EB + pz * D::xplane() + l * (8 * LP) + b;
+        for (int r = 0; r < D::R2; ++r) {
+            int line, c;
+            p.template task<8>(r, line, c);
+            if (l0 + line >= NB) continue;
+            cx<T> x[RB];
 #pragma unroll
-        for (int c = 0; c < 8; ++c) e[c * LP] = cmulc(x[c], tws[b * c]);
-    }
-    __syncthreads();
-    // x stage 2: the thread of (plane, c, pair)
-    for (int t = threadIdx.x; t < PZ * 8 * NB; t += TH) {
-        const int pz = t % PZ, c = (t / PZ) % 8, l = t / (PZ * 8);
-        const cx<T>* e = EB + pz * D::xplane() + (l * 8 + c) * LP;
-        cx<T> x[RB];
+            for (int b = 0; b < RB; ++b) x[b] = p.x(line, c, b);
+            dft<RB, -1, RB>(x);
 #pragma unroll
-        for (int b = 0; b < RB; ++b) x[b] = e[b];
-        dft<RB, -1, RB>(x);
-        cx<T>* o = ZB + (l * S + c) * PZ + pz;
-#pragma unroll
-        for (int d = 0; d < RB; ++d) o[8 * d * PZ] = x[d];
-    }
-    __syncthreads();
-    // y stage 1: the thread of (plane, kx, b); y = RB a + b, the rows of the
-    // pairs b (a = 0, 2) and b + RB (a = 1, 3)
-    for (int t = threadIdx.x; t < PZ * NX * RB; t += TH) {
-        const int pz = t % PZ, kx = (t / PZ) % NX, b = t / (PZ * NX);
-        const int mx = kx == 0 ? 0 : S - kx;
-        cx<T> x[8];
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const cx<T>* row = ZB + (b + h * RB) * S * PZ + pz;
-            const cx<T> u = row[kx * PZ], v = row[mx * PZ];
-            x[h] = {T(0.5) * (u.x + v.x), T(0.5) * (u.y - v.y)};
-            x[h + 2] = {T(0.5) * (u.y + v.y), T(0.5) * (v.x - u.x)};
+            for (int d = 0; d < RB; ++d) p.put_line(l0 + line, c + 8 * d, x[d]);
         }
-#pragma unroll
-        for (int a = 4; a < 8; ++a) x[a] = czero<T>();
-        dft<8, -1, 4>(x);
-        cx<T>* e = EB + (b * NX + kx) * PZ + pz;
-#pragma unroll
-        for (int c = 0; c < 8; ++c) e[c * RB * NX * PZ] = cmulc(x[c], tws[b * c]);
+        __syncwarp();
     }
     __syncthreads();
-    // y stage 2: the thread of (plane, kx, c) -> ky = c + 8 d
-    cx<T>* out = xy + int64_t(g) * N + z0;
-    const int64_t pitch = int64_t(n_groups) * N;   // between columns
-    for (int t = threadIdx.x; t < PZ * NX * 8; t += TH) {
-        const int pz = t % PZ, kx = (t / PZ) % NX, c = t / (PZ * NX);
-        const cx<T>* e = EB + (c * RB * NX + kx) * PZ + pz;
-        cx<T> x[RB];
+    // y: rows y = RB a + b, from the lines b (a = 0, 2) and b + RB (a = 1, 3)
+    cx<T>* out = xy + D::xy(g, 0) + D::zoff(z);
+    for (int k0 = warp * P::LINES; k0 < NX; k0 += WARPS * P::LINES) {
 #pragma unroll
-        for (int b = 0; b < RB; ++b) x[b] = e[b * NX * PZ];
-        dft<RB, -1, RB>(x);
-        cx<T>* o = out + (c * NX + kx) * pitch + pz;
+        for (int r = 0; r < D::R1; ++r) {
+            int line, b;
+            if (!p.template task<RB>(r, line, b) || k0 + line >= NX) continue;
+            cx<T> x[8];
 #pragma unroll
-        for (int d = 0; d < RB; ++d) o[8 * d * NX * pitch] = x[d];
+            for (int h = 0; h < 2; ++h) {
+                const cx<T> u = p.z(2 * h, b, k0 + line), v = p.z(2 * h + 1, b, k0 + line);
+                x[h] = {T(0.5) * (u.x + v.x), T(0.5) * (u.y - v.y)};
+                x[h + 2] = {T(0.5) * (u.y + v.y), T(0.5) * (v.x - u.x)};
+            }
+#pragma unroll
+            for (int a = 4; a < 8; ++a) x[a] = czero<T>();
+            dft<8, -1, 4>(x);
+#pragma unroll
+            for (int c = 0; c < 8; ++c) p.x(line, c, b) = cmulc(x[c], p.tw[b * c]);
+        }
+        __syncwarp();
+#pragma unroll
+        for (int r = 0; r < D::R2; ++r) {
+            int line, c;
+            p.template task<8>(r, line, c);
+            if (k0 + line >= NX) continue;
+            cx<T> x[RB];
+#pragma unroll
+            for (int b = 0; b < RB; ++b) x[b] = p.x(line, c, b);
+            dft<RB, -1, RB>(x);
+            cx<T>* o = out + ((k0 + line) * S + c) * PZ;
+#pragma unroll
+            for (int d = 0; d < RB; ++d) o[8 * d * PZ] = x[d];
+        }
+        __syncwarp();
     }
 }
 
 // ---------------------------------------------------------------------------
-// Forward z lines: N values in, S out; 32 columns per CTA (16 where 32 would
-// exceed the 48 KB of static shared memory).
-template <typename T, int NB>
+// Forward z lines, FP64: N values in, S out; 32 consecutive columns of a group
+// per CTA (16 where 32 would exceed the 48 KB of static shared memory).
+template <int NB>
 __host__ __device__ constexpr int z_lines() {
-    return sizeof(cx<T>) * (32 * size_t(Dim<T, NB>::LINE) + Dim<T, NB>::S) <= 48 * 1024 ? 32 : 16;
+    return sizeof(cx<double>) * (32 * size_t(Dim<double, NB>::LINE) + Dim<double, NB>::S) <= 48 * 1024 ? 32 : 16;
 }
-template <typename T, int NB>
-__global__ void __launch_bounds__(256) k_gz_fwd(const cx<T>* __restrict__ xy, const cx<T>* __restrict__ tw,
-                                                cx<T>* __restrict__ spec, int64_t n_lines) {
+template <int NB>
+__global__ void __launch_bounds__(256) k_gz_fwd(const cx<double>* __restrict__ xy, const cx<double>* __restrict__ tw,
+                                                cx<double>* __restrict__ spec, int n_groups) {
+    using T = double;
     using D = Dim<T, NB>;
-    constexpr int N = D::N, S = D::S, RB = D::RB, LP = D::LP, LINE = D::LINE;
-    constexpr int kZLines = z_lines<T, NB>();
-    __shared__ cx<T> e[kZLines * LINE];
+    constexpr int S = D::S, RB = D::RB, LP = D::LP, LINE = D::LINE, L = z_lines<NB>(), PER = (int(D::NC) + L - 1) / L;
+    __shared__ cx<T> e[L * LINE];
     __shared__ cx<T> tws[S];
     for (int i = threadIdx.x; i < S; i += 256) tws[i] = ld(tw + i);
     __syncthreads();
-    const int64_t first = int64_t(blockIdx.x) * kZLines;
-    for (int t = threadIdx.x; t < kZLines * RB; t += 256) {
+    const int g = blockIdx.x / PER, c0 = blockIdx.x % PER * L, n = min(L, int(D::NC) - c0);
+    for (int t = threadIdx.x; t < n * RB; t += 256) {
         const int b = t % RB, l = t / RB;
-        if (first + l >= n_lines) break;
-        const cx<T>* in = xy + (first + l) * N + b;
+        const cx<T>* in = xy + D::xy(g, c0 + l);
         cx<T> x[8];
 #pragma unroll
-        for (int a = 0; a < 4; ++a) x[a] = ld(in + RB * a);
+        for (int a = 0; a < 4; ++a) x[a] = ld(in + D::zoff(RB * a + b));
 #pragma unroll
         for (int a = 4; a < 8; ++a) x[a] = czero<T>();
         dft<8, -1, 4>(x);
@@ -201,14 +259,13 @@ __global__ void __launch_bounds__(256) k_gz_fwd(const cx<T>* __restrict__ xy, co
         for (int c = 0; c < 8; ++c) e[l * LINE + c * LP + b] = cmulc(x[c], tws[b * c]);
     }
     __syncthreads();
-    for (int t = threadIdx.x; t < kZLines * 8; t += 256) {
+    for (int t = threadIdx.x; t < n * 8; t += 256) {
         const int c = t % 8, l = t / 8;
-        if (first + l >= n_lines) break;
         cx<T> x[RB];
 #pragma unroll
         for (int b = 0; b < RB; ++b) x[b] = e[l * LINE + c * LP + b];
         dft<RB, -1, RB>(x);
-        cx<T>* o = spec + (first + l) * S + c;
+        cx<T>* o = spec + (int64_t(c0 + l) * n_groups + g) * S + c;
 #pragma unroll
         for (int d = 0; d < RB; ++d) o[8 * d] = x[d];
     }
@@ -276,7 +333,7 @@ __global__ void __launch_bounds__(Dim<double, NB>::MT)
            cx<double>* __restrict__ xy, const int4* __restrict__ sets, int n_super, int per, int n_groups) {
     using T = double;
     using D = Dim<T, NB>;
-    constexpr int N = D::N, S = D::S, RB = D::RB, LP = D::LP, COLS = D::COLS, MT = D::MT, LINE = D::LINE;
+    constexpr int S = D::S, RB = D::RB, LP = D::LP, COLS = D::COLS, MT = D::MT, LINE = D::LINE;
     constexpr int64_t NW = D::NC * S;
     __shared__ cx<T> e[8 * COLS * LINE];
     __shared__ cx<T> tws[S];
@@ -324,9 +381,9 @@ __global__ void __launch_bounds__(Dim<double, NB>::MT)
 #pragma unroll
             for (int i = 0; i < 8; ++i) x[i] = e[l * LINE + i * LP + b];
             dft<8, 1, 8>(x);
-            cx<T>* o = xy + (int64_t(col) * n_groups + g) * N + b;
+            cx<T>* o = xy + D::xy(g, col);
 #pragma unroll
-            for (int a = 0; a < 4; ++a) o[RB * a] = x[a];
+            for (int a = 0; a < 4; ++a) o[D::zoff(RB * a + b)] = x[a];
         }
     }
 }
@@ -624,7 +681,7 @@ __global__ void __launch_bounds__(ColDim<NB>::TH, 3)
             int first_col) {
     using C = ColDim<NB>;
     using D = Dim<float, NB>;
-    constexpr int N = D::N, S = D::S, COLS = C::COLS, LINE = C::LINE, TH = C::TH, UW = C::SL, VEC = kSetInts / 4;
+    constexpr int S = D::S, COLS = C::COLS, LINE = C::LINE, TH = C::TH, UW = C::SL, VEC = kSetInts / 4;
     __shared__ __align__(16) cx<float> lines[C::UNITS * 8 * COLS * LINE];   // [unit][target][column][LINE]
     __shared__ cx<float> tws[S];
     __shared__ int4 recs[TH / 32][2][VEC];
@@ -686,132 +743,136 @@ __global__ void __launch_bounds__(ColDim<NB>::TH, 3)
                               [&](int l, int b, const cx<float>(&x)[8]) {
                                   const int g = targets[l / COLS];
                                   if (g < 0) return;
-                                  cx<float>* o = out + ((col0 + l % COLS) * n_groups + g) * N + b;
+                                  cx<float>* o = out + D::xy(g, int(col0) + l % COLS);
 #pragma unroll
-                                  for (int a = 0; a < 4; ++a) o[D::RB * a] = x[a];
+                                  for (int a = 0; a < 4; ++a) o[D::zoff(D::RB * a + b)] = x[a];
                               });
         meet();
     }
 }
 
-// Forward z lines of a band of columns of every group (contiguous), as images
+// Forward z lines of a band of columns of every group, as images
 // [band column][n_groups + 1][IMG] (the last line of a column stays zero); a
-// CTA transforms some tens of them.
+// CTA transforms some tens of consecutive columns of a group.
 template <int NB>
-constexpr int image_lines() { return ColDim<NB>::LINE <= 72 ? 64 : 32; }
+__host__ __device__ constexpr int image_lines() { return ColDim<NB>::LINE <= 72 ? 64 : 32; }
 template <int NB>
-__global__ void __launch_bounds__(256) k_gz_image(const cx<float>* __restrict__ in, const cx<float>* __restrict__ tw,
-                                                  cx<float>* __restrict__ img, int64_t n_lines, int n_groups) {
+__global__ void __launch_bounds__(256) k_gz_image(const cx<float>* __restrict__ xy, const cx<float>* __restrict__ tw,
+                                                  cx<float>* __restrict__ img, int first_col, int band_cols,
+                                                  int n_groups) {
     using C = ColDim<NB>;
     using D = Dim<float, NB>;
-    constexpr int LINES = image_lines<NB>(), LINE = C::LINE, S = D::S, IMG = C::IMG;
-    __shared__ __align__(16) cx<float> e[LINES * LINE];
+    constexpr int L = image_lines<NB>(), LINE = C::LINE, S = D::S, IMG = C::IMG;
+    __shared__ __align__(16) cx<float> e[L * LINE];
     __shared__ cx<float> tws[S];
-    const int64_t first = int64_t(blockIdx.x) * LINES;
-    const int n = int(n_lines - first < LINES ? n_lines - first : LINES);
+    const int per = (band_cols + L - 1) / L, g = blockIdx.x / per, c0 = blockIdx.x % per * L, n = min(L, band_cols - c0);
     for (int i = threadIdx.x; i < S; i += 256) tws[i] = ld(tw + i);
     __syncthreads();
+    const cx<float>* in = xy + D::xy(g, first_col + c0);
     z_forward<NB, 2>(e, tws, int(threadIdx.x / 32) * Team<NB>::WARP_LINES, 8 * Team<NB>::WARP_LINES, n,
-                     [&](int l, int z) { return ld(in + (first + l) * D::N + z); });
+                     [&](int l, int z) { return ld(in + l * D::PZ + D::zoff(z)); });
     __syncthreads();
     for (int i = threadIdx.x; i < n * (IMG / 2); i += 256) {
-        const int64_t line = first + i / (IMG / 2);
-        reinterpret_cast<float4*>(img + (line + line / n_groups) * IMG)[i % (IMG / 2)] =
-            *reinterpret_cast<const float4*>(e + i / (IMG / 2) * LINE + i % (IMG / 2) * 2);
+        const int l = i / (IMG / 2), v = i % (IMG / 2);
+        reinterpret_cast<float4*>(img + (int64_t(c0 + l) * (n_groups + 1) + g) * IMG)[v] =
+            *reinterpret_cast<const float4*>(e + l * LINE + 2 * v);
     }
 }
 
 // ---------------------------------------------------------------------------
 // Inverse y and x transforms of PZ planes of a group into its blocks.
 template <typename T, int NB>
-__global__ void __launch_bounds__(Dim<T, NB>::threads()) k_gxy_inv(const cx<T>* __restrict__ xy, const int* __restrict__ blk,
-                                                                   const int* __restrict__ aux,
-                                                                   const cx<T>* __restrict__ tw, T* __restrict__ u,
-                                                                   const T* __restrict__ add, int add_n,
-                                                                   int64_t add_stride, int n_groups) {
+__global__ void __launch_bounds__(Dim<T, NB>::TH, sizeof(T) == 4 && NB <= 16 ? 4 : 1)
+    k_gxy_inv(const cx<T>* __restrict__ xy, const int* __restrict__ blk, const int* __restrict__ aux,
+              const cx<T>* __restrict__ tw, T* __restrict__ u, const T* __restrict__ add, int add_n,
+              int64_t add_stride) {
     using D = Dim<T, NB>;
-    constexpr int N = D::N, S = D::S, NX = D::NX, RB = D::RB, LP = D::LP, PZ = D::PZ, TH = D::threads();
+    using P = Plane<T, NB>;
+    constexpr int N = D::N, S = D::S, NX = D::NX, RB = D::RB, PZ = D::PZ, WARPS = D::TH / 32;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    cx<T>* ZB = reinterpret_cast<cx<T>*>(smem_raw);      // [NB pairs][S][PZ]
-    cx<T>* EB = ZB + NB * S * PZ;
-    cx<T>* tws = EB + D::exch(PZ);
-    const int g = blockIdx.x / (N / PZ), z0 = (blockIdx.x % (N / PZ)) * PZ;
-    for (int i = threadIdx.x; i < S; i += TH) tws[i] = ld(tw + i);
+    P p(smem_raw, tw);
+    const int g = blockIdx.x / (N / PZ), z = int(blockIdx.x % (N / PZ)) * PZ + p.pz, cz = z >= NB ? 4 : 0;
+    const int warp = int(threadIdx.x / 32), zl = z - (cz ? NB : 0);
     __syncthreads();
-    // y stage 1: the thread of (plane, kx, c) over ky = c + 8 d
-    const cx<T>* in = xy + int64_t(g) * N + z0;
-    const int64_t pitch = int64_t(n_groups) * N;   // between columns
-    for (int t = threadIdx.x; t < PZ * NX * 8; t += TH) {
-        const int pz = t % PZ, kx = (t / PZ) % NX, c = t / (PZ * NX);
-        const cx<T>* p = in + (c * NX + kx) * pitch + pz;
-        cx<T> x[RB];
+    // y: ky = c + 8 d -> y = RB a + b; the rows y and y + n_b (half spectra A
+    // and B of real rows) as one complex line A + i B
+    const cx<T>* in = xy + D::xy(g, 0) + D::zoff(z);
+    for (int k0 = warp * P::LINES; k0 < NX; k0 += WARPS * P::LINES) {
 #pragma unroll
-        for (int d = 0; d < RB; ++d) x[d] = ld(p + 8 * d * NX * pitch);
-        dft<RB, 1, RB>(x);
-        cx<T>* e = EB + (c * RB * NX + kx) * PZ + pz;
+        for (int r = 0; r < D::R2; ++r) {
+            int line, c;
+            p.template task<8>(r, line, c);
+            if (k0 + line >= NX) continue;
+            const cx<T>* q = in + ((k0 + line) * S + c) * PZ;
+            cx<T> x[RB];
 #pragma unroll
-        for (int b = 0; b < RB; ++b) e[b * NX * PZ] = cmulw(x[b], tws[b * c]);
-    }
-    __syncthreads();
-    // y stage 2: the thread of (plane, kx, b) -> y = RB a + b; the rows y and
-    // y + n_b (half spectra A and B of real rows) as one complex line A + i B
-    for (int t = threadIdx.x; t < PZ * NX * RB; t += TH) {
-        const int pz = t % PZ, kx = (t / PZ) % NX, b = t / (PZ * NX);
-        const cx<T>* e = EB + (b * NX + kx) * PZ + pz;
-        cx<T> x[8];
+            for (int d = 0; d < RB; ++d) x[d] = ld(q + 8 * d * PZ);
+            dft<RB, 1, RB>(x);
 #pragma unroll
-        for (int c = 0; c < 8; ++c) x[c] = e[c * RB * NX * PZ];
-        dft<8, 1, 8>(x);
-        const bool edge = kx == 0 || 2 * kx == S;   // real for a real row
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            cx<T> A = x[h], B = x[h + 2];
-            if (edge) A.y = B.y = T(0);
-            cx<T>* row = ZB + (b + h * RB) * S * PZ + pz;
-            row[kx * PZ] = {A.x - B.y, A.y + B.x};
-            if (!edge) row[(S - kx) * PZ] = {A.x + B.y, B.x - A.y};
+            for (int b = 0; b < RB; ++b) p.x(line, c, b) = cmulw(x[b], p.tw[b * c]);
         }
-    }
-    __syncthreads();
-    // x stage 1: the thread of (plane, c, pair)
-    for (int t = threadIdx.x; t < PZ * 8 * NB; t += TH) {
-        const int pz = t % PZ, c = (t / PZ) % 8, l = t / (PZ * 8);
-        const cx<T>* p = ZB + (l * S + c) * PZ + pz;
-        cx<T> x[RB];
+        __syncwarp();
 #pragma unroll
-        for (int d = 0; d < RB; ++d) x[d] = p[8 * d * PZ];
-        dft<RB, 1, RB>(x);
-        cx<T>* e = EB + pz * D::xplane() + (l * 8 + c) * LP;
+        for (int r = 0; r < D::R1; ++r) {
+            int line, b;
+            if (!p.template task<RB>(r, line, b) || k0 + line >= NX) continue;
+            const int kx = k0 + line;
+            cx<T> x[8];
 #pragma unroll
-        for (int b = 0; b < RB; ++b) e[b] = cmulw(x[b], tws[b * c]);
-    }
-    __syncthreads();
-    // x stage 2: the thread of (plane, b, pair) -> x = RB a + b of the rows
-    // y = l (real part) and l + n_b (imaginary part)
-    const int* gb = blk + int64_t(g) * 8;
-    const int* ga = aux + int64_t(g) * 8;
-    for (int t = threadIdx.x; t < PZ * RB * NB; t += TH) {
-        const int pz = t % PZ, b = (t / PZ) % RB, l = t / (PZ * RB);
-        const cx<T>* e = EB + pz * D::xplane() + l * (8 * LP) + b;
-        cx<T> x[8];
-#pragma unroll
-        for (int c = 0; c < 8; ++c) x[c] = e[c * LP];
-        dft<8, 1, 8>(x);
-        const int z = z0 + pz, cz = z >= NB ? 4 : 0, zl = z - (cz ? NB : 0);
-#pragma unroll
-        for (int ch = 0; ch < 4; ++ch) {   // child (x, y) of the plane
-            const int id = (ch & 1) + (ch & 2) + cz;
-            const int bi = __ldg(gb + id);
-            if (bi < 0) continue;
-            const int sl = add != nullptr ? __ldg(ga + id) : -1;
+            for (int c = 0; c < 8; ++c) x[c] = p.x(line, c, b);
+            dft<8, 1, 8>(x);
+            const bool edge = kx == 0 || 2 * kx == S;   // real for a real row
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
-                const int a = 2 * (ch & 1) + h, xl = RB * h + b;
-                T v = (ch & 2) ? x[a].y : x[a].x;
-                if (sl >= 0) v += __ldg(add + int64_t(sl) * add_stride + (int64_t(zl) * add_n + l) * add_n + xl);
-                u[int64_t(bi) * (NB * NB * NB) + (int64_t(zl) * NB + l) * NB + xl] = v;
+                cx<T> A = x[h], B = x[h + 2];
+                if (edge) A.y = B.y = T(0);
+                p.z(2 * h, b, kx) = {A.x - B.y, A.y + B.x};
+                p.z(2 * h + 1, b, kx) = {A.x + B.y, B.x - A.y};
             }
         }
+        __syncwarp();
+    }
+    __syncthreads();
+    // x: the rows y = l (real part) and l + n_b (imaginary part)
+    for (int l0 = warp * P::LINES; l0 < NB; l0 += WARPS * P::LINES) {
+#pragma unroll
+        for (int r = 0; r < D::R2; ++r) {
+            int line, c;
+            p.template task<8>(r, line, c);
+            if (l0 + line >= NB) continue;
+            cx<T> x[RB];
+#pragma unroll
+            for (int d = 0; d < RB; ++d) x[d] = p.line_at(l0 + line, c + 8 * d);
+            dft<RB, 1, RB>(x);
+#pragma unroll
+            for (int b = 0; b < RB; ++b) p.x(line, c, b) = cmulw(x[b], p.tw[b * c]);
+        }
+        __syncwarp();
+#pragma unroll
+        for (int r = 0; r < D::R1; ++r) {
+            int line, b;
+            if (!p.template task<RB>(r, line, b) || l0 + line >= NB) continue;
+            const int l = l0 + line;
+            cx<T> x[8];
+#pragma unroll
+            for (int c = 0; c < 8; ++c) x[c] = p.x(line, c, b);
+            dft<8, 1, 8>(x);
+#pragma unroll
+            for (int ch = 0; ch < 4; ++ch) {   // child (x, y) of the plane
+                const int id = ch + cz;
+                const int bi = __ldg(blk + int64_t(g) * 8 + id);
+                if (bi < 0) continue;
+                const int sl = add != nullptr ? __ldg(aux + int64_t(g) * 8 + id) : -1;
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const int a = 2 * (ch & 1) + h, xl = RB * h + b;
+                    T v = (ch & 2) ? x[a].y : x[a].x;
+                    if (sl >= 0) v += __ldg(add + int64_t(sl) * add_stride + (int64_t(zl) * add_n + l) * add_n + xl);
+                    u[int64_t(bi) * (NB * NB * NB) + (int64_t(zl) * NB + l) * NB + xl] = v;
+                }
+            }
+        }
+        __syncwarp();
     }
 }
 
@@ -826,13 +887,11 @@ cudaError_t GroupSize<T, NB>::forward(const GroupTables& g, const T* f, void* xy
     if (e != cudaSuccess || g.n_groups == 0) return e;
     auto* p = static_cast<dev::cx<T>*>(xy);
     const auto* tw = static_cast<const dev::cx<T>*>(g.tw);
-    k<<<unsigned(g.n_groups * (D::N / D::PZ)), D::threads(), smem, st>>>(f, g.blk, tw, p, g.n_groups);
+    k<<<unsigned(g.n_groups * (D::N / D::PZ)), D::TH, smem, st>>>(f, g.blk, tw, p);
     if ((e = cudaGetLastError()) != cudaSuccess || group_banded<T>()) return e;
     if constexpr (!group_banded<T>()) {
-        const int64_t lines = g.n_groups * D::NC;
-        constexpr int per = grp::z_lines<T, NB>();
-        grp::k_gz_fwd<T, NB><<<unsigned((lines + per - 1) / per), 256, 0, st>>>(
-            p, tw, static_cast<dev::cx<T>*>(spec), lines);
+        constexpr int L = grp::z_lines<NB>(), per = (int(D::NC) + L - 1) / L;
+        grp::k_gz_fwd<NB><<<unsigned(g.n_groups * per), 256, 0, st>>>(p, tw, static_cast<dev::cx<T>*>(spec), g.n_groups);
     }
     return cudaGetLastError();
 }
@@ -854,9 +913,8 @@ cudaError_t GroupSize<T, NB>::products(const GroupTables& g, const void* in, con
         for (int c0 = 0; c0 < nc; c0 += g.band_cols) {
             const int n = std::min(g.band_cols, nc - c0), cols = n / C::COLS;
             constexpr int L = grp::image_lines<NB>();
-            const int64_t lines = int64_t(n) * g.n_groups;
-            grp::k_gz_image<NB><<<unsigned((lines + L - 1) / L), 256, 0, st>>>(src + int64_t(c0) * g.n_groups * D::N, tw,
-                                                                              img, lines, g.n_groups);
+            grp::k_gz_image<NB><<<unsigned(g.n_groups * ((n + L - 1) / L)), 256, 0, st>>>(src, tw, img, c0, n,
+                                                                                         g.n_groups);
             if ((e = cudaGetLastError()) != cudaSuccess) return e;
             // sets per unit: one load of the kernel rows for all of them,
             // while the launch keeps some waves of CTAs
@@ -889,8 +947,8 @@ cudaError_t GroupSize<T, NB>::inverse(const GroupTables& g, const void* xy, T* u
     auto k = grp::k_gxy_inv<T, NB>;
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
     if (e != cudaSuccess || g.n_groups == 0) return e;
-    k<<<unsigned(g.n_groups * (D::N / D::PZ)), D::threads(), smem, st>>>(
-        static_cast<const dev::cx<T>*>(xy), g.blk, g.aux, static_cast<const dev::cx<T>*>(g.tw), u, add, add_n, add_stride, g.n_groups);
+    k<<<unsigned(g.n_groups * (D::N / D::PZ)), D::TH, smem, st>>>(
+        static_cast<const dev::cx<T>*>(xy), g.blk, g.aux, static_cast<const dev::cx<T>*>(g.tw), u, add, add_n, add_stride);
     return cudaGetLastError();
 }
 

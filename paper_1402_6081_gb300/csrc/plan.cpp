@@ -292,10 +292,12 @@ static lgf_status get_spectra(int device, int n_b, int S, int h, int kind, int p
                 }
                 std::vector<std::complex<double>> w(static_cast<size_t>(NW));
                 kernel_spectrum(pitch, n, h, S, d, tab->data(), V, w.data());
-                const int64_t cols = NW / S;
-                for (int64_t c = 0; c < cols; ++c) {
+                const int NX = nx_of(S);
+                // frequency kz of column c = kx S + ky
+                auto at = [&](int64_t c, int kz) { return w[size_t((int64_t(kz) * S + c % S) * NX + c / S)]; };
+                for (int64_t c = 0; c < NW / S; ++c) {
                     if (prec == LGF_FP64) {   // column by column, kz fastest
-                        for (int kz = 0; kz < S; ++kz) out_row[c * S + kz] = w[size_t(kz * cols + c)];
+                        for (int kz = 0; kz < S; ++kz) out_row[c * S + kz] = at(c, kz);
                         continue;
                     }
                     // column by column, then row by row: kz = r + 8 m by r, the m in pairs
@@ -303,8 +305,8 @@ static lgf_status get_spectra(int device, int n_b, int S, int h, int kind, int p
                     std::complex<double>* o = &all[size_t((c * kGroupRows + row) * (16 * gs.pairs))];
                     for (int r = 0; r < 8; ++r)
                         for (int j = 0; j < gs.pairs; ++j, o += 2) {
-                            const std::complex<double> a = w[size_t((r + 16 * j) * cols + c)],
-                                                       b = 2 * j + 1 < gs.rb ? w[size_t((r + 16 * j + 8) * cols + c)] : 0.0;
+                            const std::complex<double> a = at(c, r + 16 * j);
+                            const std::complex<double> b = 2 * j + 1 < gs.rb ? at(c, r + 16 * j + 8) : 0.0;
                             o[0] = {a.real(), b.real()};
                             o[1] = {a.imag(), b.imag()};
                         }
