@@ -53,28 +53,34 @@ struct GroupTables {
 struct GroupShape { int image = 0, cols = 1, rb = 0, pairs = 0; };
 GroupShape group_shape(int n_b);
 
+// early: the kernel that precedes on st (the previous phase) may still be
+// draining when this phase's first kernel starts (programmatic serialization;
+// the kernels wait for it themselves).  The forward phase waits for all prior
+// work; early there is for its own second kernel.
+//
 // One block size.  xy: n_groups * columns * N complex values (z lines of the
 // x, y transforms); FP64: spec: columns * n_groups * S.
 //   FP32: forward -> xy; products: xy -> out (as xy); inverse: out
 //   FP64: forward -> xy, then spec; products: spec -> xy; inverse: xy
 template <typename T, int NB>
 struct GroupSize {
-    static cudaError_t forward(const GroupTables& g, const T* f, void* xy, void* spec, cudaStream_t st);
-    static cudaError_t products(const GroupTables& g, const void* in, const void* kern, void* out, cudaStream_t st);
+    static cudaError_t forward(const GroupTables& g, const T* f, void* xy, void* spec, int early, cudaStream_t st);
+    static cudaError_t products(const GroupTables& g, const void* in, const void* kern, void* out, int early,
+                                cudaStream_t st);
     // inverse xy transforms into the blocks of u, plus the level-1 field add
     // (slots of add_n^3 values, add_stride apart) when given
     static cudaError_t inverse(const GroupTables& g, const void* xy, T* u, const T* add, int add_n,
-                               int64_t add_stride, cudaStream_t st);
+                               int64_t add_stride, int early, cudaStream_t st);
 };
 
 bool group_supported(int n_b);
 template <typename T>
 struct Group {
-    static cudaError_t forward(int n_b, const GroupTables& g, const T* f, void* xy, void* spec, cudaStream_t st);
+    static cudaError_t forward(int n_b, const GroupTables& g, const T* f, void* xy, void* spec, int early, cudaStream_t st);
     static cudaError_t products(int n_b, const GroupTables& g, const void* in, const void* kern, void* out,
-                                cudaStream_t st);
+                                int early, cudaStream_t st);
     static cudaError_t inverse(int n_b, const GroupTables& g, const void* xy, T* u, const T* add, int add_n,
-                               int64_t add_stride, cudaStream_t st);
+                               int64_t add_stride, int early, cudaStream_t st);
 };
 
 }  // namespace lgf

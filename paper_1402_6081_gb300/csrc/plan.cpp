@@ -1346,8 +1346,15 @@ static lgf_status solve_impl(lgf_plan_s* P, const T* f, T* u, cudaStream_t st) {
     auto record = [&](int k, cudaStream_t s) { return conc ? cudaEventRecord(P->join[k], s) : cudaSuccess; };
     auto wait = [&](cudaStream_t s, int k) { return conc ? cudaStreamWaitEvent(s, P->join[k], 0) : cudaSuccess; };
     // level-0 inverse FFT into u, plus the level-1 field add when given
+    // The grouped phases follow one another on st with nothing in between
+    // (events do when launches are timed).  Beside the long levels >= 2 chain
+    // of the run-time-size kernels, CTAs that started early and wait hold SMs
+    // that the chain needs (n_b = 24, 144^3: 873 us without, 900 with).
+    const int chain = P->ev.empty() && !(gen && Lm >= 2) ? 1 : 0;
     auto c2r0 = [&](const T* add) -> cudaError_t {
-        if (P->grouped) return Group<T>::inverse(nb, P->grp, group_banded<T>() ? lev[0].fh : lev[0].uh, u, add, nI, n3, st);
+        if (P->grouped)
+            return Group<T>::inverse(nb, P->grp, group_banded<T>() ? lev[0].fh : lev[0].uh, u, add, nI, n3,
+                                     Lm < 2 ? chain : 0, st);
         if constexpr (std::is_same_v<T, float>)
             if (P->fft_kernel == 2)
                 return c2r_cube(P->S0, nb, lev[0].uh, P->out_items, P->n_out, u, b3, add, nI, n3, P->cube_grid[1],
@@ -1462,7 +1469,7 @@ static lgf_status solve_impl(lgf_plan_s* P, const T* f, T* u, cudaStream_t st) {
     }
     // ---- level 0 on the caller's stream: forward FFT, near-field products
     e = timed(P, "r2c_level0", st, [&] {
-        if (P->grouped) return Group<T>::forward(nb, P->grp, f, lev[0].uh, lev[0].fh, st);
+        if (P->grouped) return Group<T>::forward(nb, P->grp, f, lev[0].uh, lev[0].fh, chain, st);
         if constexpr (std::is_same_v<T, float>)
             if (P->fft_kernel == 2) {
                 if (P->in_map_src != f)
@@ -1479,7 +1486,7 @@ static lgf_status solve_impl(lgf_plan_s* P, const T* f, T* u, cudaStream_t st) {
         e = timed(P, "mac_level01", st, [&] {
             if (P->grouped)
                 return Group<T>::products(nb, P->grp, group_banded<T>() ? lev[0].uh : lev[0].fh, lev[0].kh->ptr,
-                                          group_banded<T>() ? lev[0].fh : lev[0].uh, st);
+                                          group_banded<T>() ? lev[0].fh : lev[0].uh, chain, st);
             // directly behind the forward FFT on st (no event between them):
             // launched early, it stages its first coefficient chunks meanwhile
             const int early = !split && P->ev.empty() ? 1 : 0;
