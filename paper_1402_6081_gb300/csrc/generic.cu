@@ -13,11 +13,10 @@
 //    target sibling groups, the chunk's 343 coefficient rows staged once in
 //    shared memory from the half table, a warp per group at a time with the
 //    8 x 8 sibling products of each neighbour group in registers (mac_block).
-//  * Reg and Interp (Eqs. alg_reg, alg_interp): the three axis passes of an
-//    item in shared memory (a per-CTA scratch in global memory when the cubes
-//    do not fit), each sum over its row's band of the stencil matrix;
-//    compensated FP32 sums where asked.  Reg runs a CTA per (parent, child)
-//    for the x and y passes and sums the children in its z pass.
+//  * Reg and Interp (Eqs. alg_reg, alg_interp): the x and y passes by slabs of
+//    an item's planes, the z passes (Reg: of a parent's eight children) by
+//    bundles of columns; each sum over its row's band of the stencil matrix,
+//    compensated FP32 sums where asked.
 #include <algorithm>
 
 #include "kernels_impl.cuh"
@@ -31,7 +30,6 @@ using dev::ldg_cx;
 
 constexpr int kThreads = 256;
 constexpr int kLineThreads = 128;   // lines per CTA of the y / z passes
-constexpr int kRiThreads = 512;     // threads per Reg / Interp CTA
 
 // (cos, sign sin)(2 pi m / S), m < S, into shared memory
 template <typename T>
@@ -223,193 +221,215 @@ __global__ void __launch_bounds__(256) g_mac(const cx<T>* __restrict__ fh, const
     }
 }
 
-// ---- Reg and Interp: one 1D pass over a cube, value (i along the axis) =
-// sum_k M(i, k) in[k along the axis], M(i, k) = W[c][i][k] (interpolation) or
-// W[c][k][i] (its adjoint).  Every row of M is non-zero on one contiguous band
-// of k (the n_max nearest nodes of a point, or for the adjoint the points
-// whose stencils hold a node), found once per CTA (band[c][i] = lo | hi << 16).
-template <typename T>
+// ---- Reg and Interp: 1D passes, value (o along the axis) = sum_k M(o, k)
+// in[k along the axis], M(o, k) = W[c][o][k] (interpolation) or W[c][k][o]
+// (its adjoint).  Every row of M is non-zero on one contiguous band of k (the
+// n_max nearest nodes of a point, or for the adjoint the points whose stencils
+// hold a node), found once per CTA (band[c][o] = lo | hi << 16).
+//
+// The x and y passes of an item need one plane at a time, the z pass a bundle
+// of columns, so an item is cut into slabs of planes and then into bundles of
+// columns, with the planes between the two launches in a slices buffer (one
+// cube per item, L2-resident for the domains that leave SMs idle).  A CTA per
+// item, all three passes on its cubes, left half the warps out (125 KB of
+// cubes at n_I = 25: one CTA per SM) and ran 216 items in two waves.  Bound by
+// the instructions of the sums (8 per compensated term) and their setup: 144^3,
+// n_b = 24, compensated FP32, Reg 206 -> 88 us, Interp 167 -> 73 us.
+//
+// A warp takes one output index o for many lines: the weight is one broadcast
+// read for kLines terms per lane and the band is the same for all lanes.
+
+constexpr int kRiThreads = 256;
+constexpr int kLines = 4;   // lines per lane
+
+template <typename T, bool COMP>
 struct Sum {
-    T s = T(0), e = T(0);
-    __device__ __forceinline__ void add(T w, T x, bool comp) {
-        if constexpr (sizeof(T) == 4) {
-            if (comp) {
-                dev::acc_comp(s, e, w, x);
-                return;
-            }
+    T s = T(0), e = T(0);   // COMP: sum and its error; else two partial sums (two chains in flight)
+    __device__ __forceinline__ void add(T w, T x, int k) {
+        if constexpr (COMP) {
+            dev::acc_comp(s, e, w, x);
+        } else {
+            T& a = k & 1 ? e : s;
+            a = fma(w, x, a);
         }
-        s = fma(w, x, s);
     }
     __device__ __forceinline__ T get() const { return s + e; }
 };
 
+// one output of LINES lines of a lane: line j's value k at in[at[j] + k * st]
+template <typename T, bool COMP, int LINES>
+__device__ __forceinline__ void lines(Sum<T, COMP> (&acc)[LINES], const T* in, const int (&at)[LINES], int st,
+                                      const T* w, int wstep, int lo, int hi) {
+    int k = lo;
+    for (; k + 1 < hi; k += 2) {
+        const T w0 = w[k * wstep], w1 = w[(k + 1) * wstep];
+#pragma unroll
+        for (int j = 0; j < LINES; ++j) {
+            acc[j].add(w0, in[at[j] + k * st], 0);
+            acc[j].add(w1, in[at[j] + (k + 1) * st], 1);
+        }
+    }
+    if (k < hi) {
+#pragma unroll
+        for (int j = 0; j < LINES; ++j) acc[j].add(w[k * wstep], in[at[j] + k * st], 0);
+    }
+}
+
 // W (2 x n x n) and the bands of M for both children into shared memory
-template <typename T>
-__device__ void load_stencil(T* W_s, int* band, const T* __restrict__ W, int n, bool adjoint) {
-    for (int i = threadIdx.x; i < 2 * n * n; i += blockDim.x) W_s[i] = __ldg(W + i);
+template <typename T, bool ADJ>
+__device__ void load_stencil(T* W_s, int* band, const T* __restrict__ W, int n) {
+    for (int i = threadIdx.x; i < 2 * n * n; i += kRiThreads) W_s[i] = __ldg(W + i);
     __syncthreads();
-    for (int q = threadIdx.x; q < 2 * n; q += blockDim.x) {
-        const int c = q / n, i = q % n;
+    const int lane = threadIdx.x & 31;
+    for (int q = threadIdx.x / 32; q < 2 * n; q += kRiThreads / 32) {
+        const int c = q / n, o = q % n;
         const T* Wc = W_s + c * n * n;
-        int lo = n, hi = 0;
-        for (int k = 0; k < n; ++k)
-            if ((adjoint ? Wc[k * n + i] : Wc[i * n + k]) != T(0)) {
-                lo = min(lo, k);
-                hi = k + 1;
-            }
-        band[q] = lo < hi ? (lo | (hi << 16)) : 0;
+        auto live = [&](int k) { return k < n && (ADJ ? Wc[k * n + o] : Wc[o * n + k]) != T(0); };
+        const unsigned long long m = uint64_t(__ballot_sync(~0u, live(lane))) |
+                                     uint64_t(__ballot_sync(~0u, live(lane + 32))) << 32;
+        if (lane == 0) band[q] = m == 0 ? 0 : (__ffsll(int64_t(m)) - 1) | ((64 - __clzll(int64_t(m))) << 16);
     }
     __syncthreads();
 }
 
-// axis a of a cube of edge n (in: edge in_n <= n, zero beyond); emit(i, value).
-// Plain sums alternate two partial sums (two chains in flight).
-template <typename T, typename Emit>
-__device__ __forceinline__ void pass(const T* in, int in_n, int n, int axis, const T* Wc, const int* band,
-                                     bool adjoint, bool comp, Emit emit) {
-    const int n3 = n * n * n;
-    for (int i = threadIdx.x; i < n3; i += blockDim.x) {
-        const int x = i % n, y = (i / n) % n, z = i / (n * n);
-        const int o = axis == 0 ? x : axis == 1 ? y : z;
-        const int b = band[o];
-        const int lo = b & 0xffff, hi = min(b >> 16, in_n);
-        T v = T(0);
-        const bool live = (axis == 0 || x < in_n) && (axis == 1 || y < in_n) && (axis == 2 || z < in_n);
-        if (live) {
-            const int st = axis == 0 ? 1 : axis == 1 ? in_n : in_n * in_n;
-            const int base = axis == 0 ? (z * in_n + y) * in_n : axis == 1 ? z * in_n * in_n + x : y * in_n + x;
-            // M(o, k) = W[c][o][k] (interpolation) or W[c][k][o] (adjoint)
-            const T* wp = Wc + (adjoint ? o : o * n);
-            const int wstep = adjoint ? n : 1;
-            if (comp) {
-                Sum<T> acc;
-                for (int k = lo; k < hi; ++k) acc.add(wp[k * wstep], in[base + k * st], true);
-                v = acc.get();
-            } else {
-                T a0 = T(0), a1 = T(0);
-                int k = lo;
-                for (; k + 1 < hi; k += 2) {
-                    a0 = fma(wp[k * wstep], in[base + k * st], a0);
-                    a1 = fma(wp[(k + 1) * wstep], in[base + (k + 1) * st], a1);
-                }
-                if (k < hi) a0 = fma(wp[k * wstep], in[base + k * st], a0);
-                v = a0 + a1;
-            }
-        }
-        emit(i, v);
+// bytes of W and the bands, and the planes of a slab (its lines: kLines per lane)
+template <typename T>
+__host__ __device__ size_t stencil_bytes(int n) {
+    return (sizeof(T) * 2 * n * n + sizeof(int) * 2 * n + 15) / 16 * 16;
+}
+__host__ __device__ constexpr int slab_planes(int n) { return 32 * kLines / n; }
+
+// x and y passes of a slab of planes of item q: child c = q & 7 (Reg: 8 items
+// per parent) or slot[q] & 7 (Interp), the cube source[q] of src (edge in_n =
+// NI, or NI - 1 and zero beyond), none where that is < 0.  Planes of NI (odd)
+// rows of NI values: no bank conflicts along either axis.
+template <typename T, bool ADJ, bool COMP>
+__global__ void __launch_bounds__(kRiThreads) g_planes(const T* __restrict__ src, int in_n,
+                                                       const int* __restrict__ source, const int* __restrict__ slot,
+                                                       int slabs, const T* __restrict__ W, int NI,
+                                                       T* __restrict__ slices) {
+    extern __shared__ __align__(16) unsigned char g_smem[];
+    const int N2 = NI * NI, P = slab_planes(NI);
+    T* W_s = reinterpret_cast<T*>(g_smem);
+    int* band = reinterpret_cast<int*>(W_s + 2 * N2);
+    T* t1 = reinterpret_cast<T*>(g_smem + stencil_bytes<T>(NI));
+    T* t2 = t1 + P * N2;
+    const int q = blockIdx.x / slabs, z0 = (blockIdx.x % slabs) * P, np = min(P, in_n - z0);
+    const int s = source[q];
+    if (s < 0) return;   // uniform over the CTA
+    const int c = slot ? slot[q] & 7 : q & 7;
+    const T* in = src + (int64_t(s) * in_n + z0) * in_n * in_n;
+    for (int i = threadIdx.x; i < np * N2; i += kRiThreads) {
+        const int x = i % NI, r = i / NI, y = r % NI, z = r / NI;
+        t1[i] = x < in_n && y < in_n ? __ldg(in + (z * in_n + y) * in_n + x) : T(0);
+    }
+    load_stencil<T, ADJ>(W_s, band, W, NI);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x / 32, rows = np * NI;
+    int at[kLines];
+#pragma unroll
+    for (int j = 0; j < kLines; ++j) at[j] = min(lane + 32 * j, rows - 1) * NI;
+    const int cx_ = c & 1, cy_ = (c >> 1) & 1, wstep = ADJ ? NI : 1;
+    for (int o = warp; o < NI; o += kRiThreads / 32) {   // x: rows
+        Sum<T, COMP> acc[kLines];
+        const int b = band[cx_ * NI + o];
+        lines<T, COMP, kLines>(acc, t1, at, 1, W_s + cx_ * N2 + (ADJ ? o : o * NI), wstep, b & 0xffff, b >> 16);
+#pragma unroll
+        for (int j = 0; j < kLines; ++j)
+            if (lane + 32 * j < rows) t2[at[j] + o] = acc[j].get();
+    }
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < kLines; ++j) {
+        const int l = min(lane + 32 * j, rows - 1);
+        at[j] = l / NI * N2 + l % NI;
+    }
+    T* out = slices + (int64_t(q) * NI + z0) * N2;
+    for (int o = warp; o < NI; o += kRiThreads / 32) {   // y: columns of a plane
+        Sum<T, COMP> acc[kLines];
+        const int b = band[cy_ * NI + o];
+        lines<T, COMP, kLines>(acc, t2, at, NI, W_s + cy_ * N2 + (ADJ ? o : o * NI), wstep, b & 0xffff, b >> 16);
+#pragma unroll
+        for (int j = 0; j < kLines; ++j)
+            if (lane + 32 * j < rows) out[at[j] + o * NI] = acc[j].get();
     }
 }
 
-// a cube of len values from global memory into shared memory (or scratch)
-template <typename T>
-__device__ __forceinline__ void stage(T* dst, const T* __restrict__ src, int len) {
-    for (int i = threadIdx.x; i < len; i += blockDim.x) dst[i] = src[i];
-}
-
-// shared-memory layout of g_reg / g_interp: W, bands, then (when they fit)
-// the two intermediate cubes
-template <typename T>
-struct RiSmem {
-    __host__ __device__ static size_t head(int n) { return (sizeof(T) * 2 * n * n + sizeof(int) * 2 * n + 15) / 16 * 16; }
-    __host__ __device__ static size_t cubes(int n) { return sizeof(T) * 2 * size_t(n) * n * n; }
-};
-
-// Reg in two launches.  g_reg_xy: a CTA per (parent, child) item takes the
-// child's x and y passes (Eq. alg_reg, W_c^T along x then y) into the item's
-// slice of the slices buffer (n_parents x 8 cubes of n_I^3).  g_reg_z: a
-// thread per parent value sums, children in order, the z passes of the
-// present children's slices.
-template <typename T>
-__global__ void __launch_bounds__(kRiThreads) g_reg_xy(const T* __restrict__ child_src, int child_is_block,
-                                                       const int* __restrict__ child_index, int n_parents,
-                                                       const T* __restrict__ W, int NI, int comp,
-                                                       T* __restrict__ slices, T* __restrict__ scratch,
-                                                       int cubes_in_smem) {
+// Reg's z pass: a CTA per parent and 32 columns sums the present children's
+// slices (planes below in_n), children in order.
+template <typename T, bool COMP>
+__global__ void __launch_bounds__(kRiThreads) g_reg_z(const int* __restrict__ child_index,
+                                                      const int* __restrict__ parent_slot, int in_n, int bundles,
+                                                      T* __restrict__ dst, const T* __restrict__ W, int NI,
+                                                      const T* __restrict__ slices) {
     extern __shared__ __align__(16) unsigned char g_smem[];
-    const int NB = NI - 1, N3 = NI * NI * NI;
+    const int N2 = NI * NI, N3 = N2 * NI;
     T* W_s = reinterpret_cast<T*>(g_smem);
-    int* band = reinterpret_cast<int*>(W_s + 2 * NI * NI);
-    T* t1 = cubes_in_smem ? reinterpret_cast<T*>(g_smem + RiSmem<T>::head(NI))
-                          : scratch + int64_t(blockIdx.x) * 2 * N3;
-    T* t2 = t1 + N3;
-    load_stencil(W_s, band, W, NI, true);
-    for (int q = blockIdx.x; q < n_parents * 8; q += gridDim.x) {
-        const int s = child_index[q], c = q & 7;
-        if (s < 0) continue;                            // uniform over the CTA
-        const int cx_ = c & 1, cy_ = (c >> 1) & 1;
-        const int in_n = child_is_block ? NB : NI;
-        stage(t2, child_is_block ? child_src + int64_t(s) * NB * NB * NB : child_src + int64_t(s) * N3,
-              in_n * in_n * in_n);
-        __syncthreads();
-        pass(t2, in_n, NI, 0, W_s + cx_ * NI * NI, band + cx_ * NI, true, comp != 0, [&](int i, T v) { t1[i] = v; });
-        __syncthreads();
-        T* out = slices + int64_t(q) * N3;
-        pass(t1, NI, NI, 1, W_s + cy_ * NI * NI, band + cy_ * NI, true, comp != 0, [&](int i, T v) { out[i] = v; });
-        __syncthreads();
-    }
-}
-
-template <typename T>
-__global__ void __launch_bounds__(kThreads) g_reg_z(const int* __restrict__ child_index,
-                                                    const int* __restrict__ parent_slot, int n_parents,
-                                                    T* __restrict__ dst, const T* __restrict__ W, int NI, int comp,
-                                                    const T* __restrict__ slices) {
-    extern __shared__ __align__(16) unsigned char g_smem[];
-    const int N3 = NI * NI * NI;
-    T* W_s = reinterpret_cast<T*>(g_smem);
-    int* band = reinterpret_cast<int*>(W_s + 2 * NI * NI);
-    load_stencil(W_s, band, W, NI, true);
-    const int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (i >= int64_t(n_parents) * N3) return;
-    const int p = int(i / N3), e = int(i % N3);
-    const int xy = e % (NI * NI), z = e / (NI * NI);
-    Sum<T> acc;
+    int* band = reinterpret_cast<int*>(W_s + 2 * N2);
+    T* t = reinterpret_cast<T*>(g_smem + stencil_bytes<T>(NI));   // [child][k][32]
+    const int p = blockIdx.x / bundles, lane = threadIdx.x & 31, warp = threadIdx.x / 32;
+    const int col = (blockIdx.x % bundles) * 32 + lane, colc = min(col, N2 - 1);
     for (int c = 0; c < 8; ++c) {
-        if (child_index[int64_t(p) * 8 + c] < 0) continue;
-        const int cz_ = c >> 2;
-        const int b = band[cz_ * NI + z];
-        const T* Wc = W_s + cz_ * NI * NI;
-        const T* in = slices + (int64_t(p) * 8 + c) * N3 + xy;
-        for (int k = b & 0xffff; k < (b >> 16); ++k) acc.add(Wc[k * NI + z], in[int64_t(k) * NI * NI], comp != 0);
+        if (child_index[p * 8 + c] < 0) continue;
+        const T* in = slices + (int64_t(p) * 8 + c) * N3 + colc;
+#pragma unroll 4
+        for (int k = warp; k < in_n; k += kRiThreads / 32) t[(c * NI + k) * 32 + lane] = in[k * N2];
     }
-    dst[int64_t(parent_slot[p]) * N3 + e] = acc.get();
+    load_stencil<T, true>(W_s, band, W, NI);
+    T* out = dst + int64_t(parent_slot[p]) * N3 + col;
+    for (int o = warp; o < NI; o += kRiThreads / 32) {
+        Sum<T, COMP> acc[1];
+        for (int c = 0; c < 8; ++c) {
+            if (child_index[p * 8 + c] < 0) continue;
+            const int cz_ = c >> 2, b = band[cz_ * NI + o];
+            const int at[1] = {c * NI * 32 + lane};
+            lines<T, COMP, 1>(acc, t, at, 32, W_s + cz_ * N2 + o, NI, b & 0xffff, min(b >> 16, in_n));
+        }
+        if (col < N2) out[o * N2] = acc[0].get();
+    }
 }
 
-template <typename T>
-__global__ void __launch_bounds__(kRiThreads) g_interp(const int* __restrict__ slot, const int* __restrict__ parent,
-                                                     int n_items, T* __restrict__ u, const T* __restrict__ up,
-                                                     const T* __restrict__ W, int NI, int accumulate,
-                                                     const int* __restrict__ block, int comp,
-                                                     T* __restrict__ scratch, int cubes_in_smem) {
+// Interp's z pass: a CTA per item and 32 kLines columns, into the child's cube
+// of u or (block != nullptr) added to its first NI - 1 nodes per axis in u's
+// block.
+template <typename T, bool COMP>
+__global__ void __launch_bounds__(kRiThreads) g_interp_z(const int* __restrict__ slot, int bundles,
+                                                         T* __restrict__ u, const T* __restrict__ W, int NI,
+                                                         int accumulate, const int* __restrict__ block,
+                                                         const T* __restrict__ slices) {
     extern __shared__ __align__(16) unsigned char g_smem[];
-    const int NB = NI - 1, N3 = NI * NI * NI;
+    constexpr int kCols = 32 * kLines;
+    const int NB = NI - 1, N2 = NI * NI, N3 = N2 * NI;
     T* W_s = reinterpret_cast<T*>(g_smem);
-    int* band = reinterpret_cast<int*>(W_s + 2 * NI * NI);
-    T* t1 = cubes_in_smem ? reinterpret_cast<T*>(g_smem + RiSmem<T>::head(NI))
-                          : scratch + int64_t(blockIdx.x) * 2 * N3;
-    T* t2 = t1 + N3;
-    load_stencil(W_s, band, W, NI, false);
-    for (int it = blockIdx.x; it < n_items; it += gridDim.x) {
-        const int s = slot[it], c = s & 7;
-        const int cx_ = c & 1, cy_ = (c >> 1) & 1, cz_ = c >> 2;
-        stage(t2, up + int64_t(parent[it]) * N3, N3);
-        __syncthreads();
-        pass(t2, NI, NI, 0, W_s + cx_ * NI * NI, band + cx_ * NI, false, comp != 0, [&](int i, T v) { t1[i] = v; });
-        __syncthreads();
-        pass(t1, NI, NI, 1, W_s + cy_ * NI * NI, band + cy_ * NI, false, comp != 0, [&](int i, T v) { t2[i] = v; });
-        __syncthreads();
-        if (block) {
-            T* o = u + int64_t(block[it]) * NB * NB * NB;
-            pass(t2, NI, NI, 2, W_s + cz_ * NI * NI, band + cz_ * NI, false, comp != 0, [&](int i, T v) {
-                const int x = i % NI, y = (i / NI) % NI, z = i / (NI * NI);
-                if (x < NB && y < NB && z < NB) o[(z * NB + y) * NB + x] += v;
-            });
-        } else {
-            T* o = u + int64_t(s) * N3;
-            pass(t2, NI, NI, 2, W_s + cz_ * NI * NI, band + cz_ * NI, false, comp != 0,
-                 [&](int i, T v) { o[i] = accumulate ? o[i] + v : v; });
+    int* band = reinterpret_cast<int*>(W_s + 2 * N2);
+    T* t = reinterpret_cast<T*>(g_smem + stencil_bytes<T>(NI));   // [k][kCols]
+    const int it = blockIdx.x / bundles, col0 = (blockIdx.x % bundles) * kCols;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x / 32;
+    const T* in = slices + int64_t(it) * N3;
+#pragma unroll 4
+    for (int i = threadIdx.x; i < NI * kCols; i += kRiThreads)
+        t[i] = in[(i / kCols) * N2 + min(col0 + i % kCols, N2 - 1)];
+    load_stencil<T, false>(W_s, band, W, NI);
+    const int s = slot[it], cz_ = (s >> 2) & 1;
+    int at[kLines], to[kLines];   // to: the column's place in the output, < 0: none
+#pragma unroll
+    for (int j = 0; j < kLines; ++j) {
+        at[j] = lane + 32 * j;
+        const int col = col0 + at[j], x = col % NI, y = col / NI;
+        to[j] = block ? (x < NB && y < NB ? y * NB + x : -1) : (col < N2 ? col : -1);
+    }
+    const int nz = block ? NB : NI, step = block ? NB * NB : N2;
+    T* out = block ? u + int64_t(block[it]) * NB * NB * NB : u + int64_t(s) * N3;
+    const bool add = block || accumulate;
+    for (int o = warp; o < nz; o += kRiThreads / 32) {
+        Sum<T, COMP> acc[kLines];
+        const int b = band[cz_ * NI + o];
+        lines<T, COMP, kLines>(acc, t, at, kCols, W_s + cz_ * N2 + o * NI, 1, b & 0xffff, b >> 16);
+#pragma unroll
+        for (int j = 0; j < kLines; ++j) {
+            if (to[j] < 0) continue;
+            T* v = out + to[j] + o * step;
+            *v = add ? *v + acc[j].get() : acc[j].get();
         }
-        __syncthreads();
     }
 }
 
@@ -517,46 +537,69 @@ cudaError_t Generic<T>::mac(const void* fh, const void* kh, void* uh, const int*
     return cudaGetLastError();
 }
 
-// Reg / Interp: W and its bands in shared memory, and the two intermediate
-// cubes too when they fit (else the CTA's 2 n_I^3 slice of the scratch)
-template <typename T>
-static size_t ri_smem(int NI, int* cubes_in_smem) {
-    const size_t head = gen::RiSmem<T>::head(NI), cubes = gen::RiSmem<T>::cubes(NI);
-    *cubes_in_smem = head + cubes <= 200 * 1024 ? 1 : 0;
-    return head + (*cubes_in_smem ? cubes : 0);
+template <typename T, bool ADJ, bool COMP>
+static cudaError_t launch_planes(const T* src, int in_n, const int* source, const int* slot, int n_items, const T* W,
+                                 int NI, T* slices, cudaStream_t st) {
+    const int P = gen::slab_planes(NI), slabs = (in_n + P - 1) / P;
+    const size_t smem = gen::stencil_bytes<T>(NI) + sizeof(T) * 2 * P * NI * NI;
+    auto k = gen::g_planes<T, ADJ, COMP>;
+    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+    if (e != cudaSuccess) return e;
+    k<<<unsigned(int64_t(n_items) * slabs), gen::kRiThreads, smem, st>>>(src, in_n, source, slot, slabs, W, NI, slices);
+    return cudaGetLastError();
+}
+
+template <typename T, bool COMP>
+static cudaError_t launch_reg(int NI, const T* src, int in_n, const int* child_index, const int* parent_slot,
+                              int n_parents, T* dst, const T* W, T* slices, cudaStream_t st) {
+    cudaError_t e = launch_planes<T, true, COMP>(src, in_n, child_index, nullptr, 8 * n_parents, W, NI, slices, st);
+    if (e != cudaSuccess) return e;
+    const int bundles = (NI * NI + 31) / 32;
+    const size_t smem = gen::stencil_bytes<T>(NI) + sizeof(T) * 8 * NI * 32;
+    auto k = gen::g_reg_z<T, COMP>;
+    if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem))) != cudaSuccess) return e;
+    k<<<unsigned(int64_t(n_parents) * bundles), gen::kRiThreads, smem, st>>>(child_index, parent_slot, in_n, bundles,
+                                                                            dst, W, NI, slices);
+    return cudaGetLastError();
+}
+
+template <typename T, bool COMP>
+static cudaError_t launch_interp(int NI, const int* slot, const int* parent, int n_items, T* u, const T* up,
+                                 const T* W, int accumulate, const int* block, T* slices, cudaStream_t st) {
+    cudaError_t e = launch_planes<T, false, COMP>(up, NI, parent, slot, n_items, W, NI, slices, st);
+    if (e != cudaSuccess) return e;
+    const int cols = 32 * gen::kLines, bundles = (NI * NI + cols - 1) / cols;
+    const size_t smem = gen::stencil_bytes<T>(NI) + sizeof(T) * NI * cols;
+    auto k = gen::g_interp_z<T, COMP>;
+    if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem))) != cudaSuccess) return e;
+    k<<<unsigned(int64_t(n_items) * bundles), gen::kRiThreads, smem, st>>>(slot, bundles, u, W, NI, accumulate, block,
+                                                                          slices);
+    return cudaGetLastError();
 }
 
 template <typename T>
 cudaError_t Generic<T>::reg(int n_b, const T* child_src, int child_is_block, const int* child_index,
-                            const int* parent_slot, int n_parents, T* dst, const T* W_dev, int comp, T* scratch,
-                            T* slices, int n_ctas, cudaStream_t st) {
+                            const int* parent_slot, int n_parents, T* dst, const T* W_dev, int comp, T* slices,
+                            cudaStream_t st) {
     if (n_parents == 0) return cudaSuccess;
-    const int NI = n_b + 1;
-    int in_smem = 0;
-    const size_t smem = ri_smem<T>(NI, &in_smem);
-    cudaError_t e = cudaFuncSetAttribute(gen::g_reg_xy<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
-    if (e != cudaSuccess) return e;
-    const int items = 8 * n_parents;
-    gen::g_reg_xy<T><<<in_smem ? items : std::min(items, n_ctas), gen::kRiThreads, smem, st>>>(
-        child_src, child_is_block, child_index, n_parents, W_dev, NI, comp, slices, scratch, in_smem);
-    const size_t smem_z = gen::RiSmem<T>::head(NI);
-    gen::g_reg_z<T><<<gen::grid_for(int64_t(n_parents) * NI * NI * NI), gen::kThreads, smem_z, st>>>(
-        child_index, parent_slot, n_parents, dst, W_dev, NI, comp, slices);
-    return cudaGetLastError();
+    const int NI = n_b + 1, in_n = child_is_block ? n_b : NI;
+    if constexpr (sizeof(T) == 4)
+        if (comp)
+            return launch_reg<T, true>(NI, child_src, in_n, child_index, parent_slot, n_parents, dst, W_dev, slices,
+                                       st);
+    return launch_reg<T, false>(NI, child_src, in_n, child_index, parent_slot, n_parents, dst, W_dev, slices, st);
 }
 
 template <typename T>
 cudaError_t Generic<T>::interp(int n_b, const int* slot, const int* parent, int n_items, T* u, const T* up,
-                               const T* W_dev, int accumulate, const int* block, int comp, T* scratch, int n_ctas,
+                               const T* W_dev, int accumulate, const int* block, int comp, T* slices,
                                cudaStream_t st) {
     if (n_items == 0) return cudaSuccess;
-    int in_smem = 0;
-    const size_t smem = ri_smem<T>(n_b + 1, &in_smem);
-    cudaError_t e = cudaFuncSetAttribute(gen::g_interp<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
-    if (e != cudaSuccess) return e;
-    gen::g_interp<T><<<in_smem ? n_items : std::min(n_items, n_ctas), gen::kRiThreads, smem, st>>>(
-        slot, parent, n_items, u, up, W_dev, n_b + 1, accumulate, block, comp, scratch, in_smem);
-    return cudaGetLastError();
+    const int NI = n_b + 1;
+    if constexpr (sizeof(T) == 4)
+        if (comp)
+            return launch_interp<T, true>(NI, slot, parent, n_items, u, up, W_dev, accumulate, block, slices, st);
+    return launch_interp<T, false>(NI, slot, parent, n_items, u, up, W_dev, accumulate, block, slices, st);
 }
 
 template struct Generic<float>;

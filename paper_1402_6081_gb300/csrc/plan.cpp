@@ -431,13 +431,11 @@ struct lgf_plan_s {
     int symmetric_spectra = 0;          // option: 1 = reflection-reduced interval tables
     // block sizes without per-size kernels: the run-time-size kernels, their
     // twiddle tables (per transform length), the stencils in device memory
-    // (per parent level) and the Reg / Interp scratch (n_ctas x 3 n_I^3 each)
+    // (per parent level) and the Reg / Interp slices (a cube per child)
     bool generic = false;
     std::map<int, void*> tw_dev;
     std::vector<void*> W_dev;
-    void* gscratch[2] = {nullptr, nullptr};
-    void* gslices = nullptr;   // Reg's per-child cubes (run-time-size kernels)
-    int gctas = 0;
+    void* gslices = nullptr;
     int mac_gpc = 0;                    // option: sibling groups per CTA of the one-CTA-per-chunk products
     int cube_grid[2] = {0, 0};
     int* fft_ctr = nullptr;
@@ -1249,18 +1247,13 @@ static lgf_status build_plan(lgf_plan_s* P, const std::vector<HostPlan>& hp) {
                 LGF_OK)
                 return s;
         }
-        // Reg / Interp scratch: two CTAs per SM, 2 cubes of n_I^3 each, and
-        // Reg's slices for the largest level (8 per parent)
+        // Reg's and Interp's slices, a cube per child of the largest level
+        // (both run on one stream, one launch after the other)
         if (Lmac >= 2) {
-            int n_sm = 0;
-            LGF_CUDA(cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, P->device));
-            P->gctas = 2 * n_sm;
-            const size_t bytes = size_t(P->gctas) * 2 * n3 * elem;
-            for (void*& g : P->gscratch)
-                if ((s = dalloc(P, bytes, &g, false)) != LGF_OK) return s;
-            size_t parents = 0;
-            for (int l = 2; l <= Lmac; ++l) parents = std::max(parents, size_t(P->lev[size_t(l)].n_reg));
-            if ((s = dalloc(P, parents * 8 * n3 * elem, &P->gslices, false)) != LGF_OK) return s;
+            size_t cubes = 0;
+            for (int l = 2; l <= Lmac; ++l)
+                cubes = std::max({cubes, 8 * size_t(P->lev[size_t(l)].n_reg), size_t(P->lev[size_t(l) - 1].n_int)});
+            if ((s = dalloc(P, cubes * n3 * elem, &P->gslices, false)) != LGF_OK) return s;
         }
     }
     return ok();
@@ -1321,14 +1314,14 @@ static lgf_status solve_impl(lgf_plan_s* P, const T* f, T* u, cudaStream_t st) {
                       const T* W, int comp, cudaStream_t s) {
         if (gen)
             return Gn::reg(nb, src, from_blocks, child, parent, n, dst, static_cast<const T*>(P->W_dev[size_t(l)]),
-                           comp, static_cast<T*>(P->gscratch[0]), static_cast<T*>(P->gslices), P->gctas, s);
+                           comp, static_cast<T*>(P->gslices), s);
         return Lc::reg(nb, nm, src, from_blocks, child, parent, n, dst, W, comp, s);
     };
     auto interp_of = [&](int lp, int nm, const int* slot, const int* parent, int n, T* out, const T* up, const T* W,
                          int accumulate, const int* block, int comp, cudaStream_t s) {
         if (gen)
             return Gn::interp(nb, slot, parent, n, out, up, static_cast<const T*>(P->W_dev[size_t(lp)]), accumulate,
-                              block, comp, static_cast<T*>(P->gscratch[1]), P->gctas, s);
+                              block, comp, static_cast<T*>(P->gslices), s);
         return Lc::interp(nb, nm, slot, parent, n, out, up, W, accumulate, block, comp, s);
     };
     cudaError_t e;
