@@ -201,8 +201,10 @@ struct Generic {
     static cudaError_t c2r(int S, int n_out, const void* spec, const C2RItem* items, int n_items, void* scratch,
                            T* dst, int64_t dst_stride, const T* add, int add_n, int64_t add_stride, const void* twt,
                            cudaStream_t st);
-    static cudaError_t mac(const void* fh, const void* kh, void* uh, const int* gnbr, int n_groups, int S,
-                           int include_self, cudaStream_t st);
+    // kh: chunk by chunk (get_spectra); mask: per group, the children that have
+    // a spectrum
+    static cudaError_t mac(const void* fh, const void* kh, void* uh, const int* gnbr, const int* mask, int n_groups,
+                           int S, int include_self, cudaStream_t st);
     static cudaError_t reg(int n_b, const T* child_src, int child_is_block, const int* child_index,
                            const int* parent_slot, int n_parents, T* dst, const T* W_dev, int comp, T* slices,
                            cudaStream_t st);

@@ -127,10 +127,10 @@ struct SpecEntry {
 };
 
 struct SpecKey {
-    int device, n_b, S, h, near, prec, oct;
+    int device, n_b, S, h, near, prec, form;
     bool operator<(const SpecKey& o) const {
-        return std::tie(device, n_b, S, h, near, prec, oct) <
-               std::tie(o.device, o.n_b, o.S, o.h, o.near, o.prec, o.oct);
+        return std::tie(device, n_b, S, h, near, prec, form) <
+               std::tie(o.device, o.n_b, o.S, o.h, o.near, o.prec, o.form);
     }
 };
 
@@ -223,13 +223,17 @@ static std::map<SpecKey, std::weak_ptr<SpecEntry>> g_spec_cache;
 // group.h)
 enum SpecKind { kNear = 0, kInterval = 1, kBlock = 2, kGroup = 3 };
 
-// oct (343-offset kinds only): store the 40 representatives of the offsets
-// under the reflections of G instead of the 172-row half table (the products
-// kernel maps each offset's frequencies onto its representative's)
+// Forms of the 343-offset kinds' tables: kRows the 172-row half table; kOct the
+// 40 representatives of the offsets under the reflections of G (the products
+// kernel maps each offset's frequencies onto its representative's); kChunks the
+// half table as [chunk of 32 frequencies][172][32], for the kernels that stage
+// one chunk's rows at a time
+enum TableForm { kRows = 0, kOct = 1, kChunks = 2 };
 static lgf_status get_spectra(int device, int n_b, int S, int h, int kind, int prec,
-                              std::shared_ptr<SpecEntry>& out, int oct = 0) {
-    if (kind == kNear || kind == kGroup) oct = 0;
-    const SpecKey key{device, n_b, S, h, kind, prec, oct};
+                              std::shared_ptr<SpecEntry>& out, TableForm form = kRows) {
+    if (kind == kNear || kind == kGroup) form = kRows;
+    const bool oct = form == kOct, chunked = form == kChunks;
+    const SpecKey key{device, n_b, S, h, kind, prec, form};
     std::lock_guard<std::mutex> lock(g_spec_mu);
     auto it = g_spec_cache.find(key);
     if (it != g_spec_cache.end()) {
@@ -314,6 +318,13 @@ static lgf_status get_spectra(int device, int n_b, int S, int h, int kind, int p
             }
         });
     for (auto& t : th) t.join();
+    if (chunked) {   // NWS is a multiple of 32
+        std::vector<std::complex<double>> c(all.size());
+        for (int row = 0; row < nd; ++row)
+            for (int64_t w = 0; w < NWS; w += 32)
+                std::copy_n(&all[size_t(row) * NWS + w], 32, &c[size_t(w / 32 * nd + row) * 32]);
+        all.swap(c);
+    }
     auto e = std::make_shared<SpecEntry>();
     e->device = device;
     const size_t elem = prec == LGF_FP64 ? sizeof(double) : sizeof(float);
@@ -334,7 +345,7 @@ static lgf_status get_spectra(int device, int n_b, int S, int h, int kind, int p
         ce = cudaMemcpy(e->ptr, f.data(), e->bytes, cudaMemcpyHostToDevice);
     }
     if (ce != cudaSuccess) return cuda_fail(ce, "spectra upload");
-    e->has_tmap = !near && !group && !oct && encode_table_map(*e, nd, NWS, prec);
+    e->has_tmap = !near && !group && form == kRows && encode_table_map(*e, nd, NWS, prec);
     g_spec_cache[key] = e;
     out = e;
     return ok();
@@ -385,6 +396,7 @@ struct DevLevel {
     void* ft = nullptr;
     void* ut = nullptr;
     int* gnbr = nullptr;
+    int* gmask = nullptr;   // children with a spectrum, a bit each (run-time-size products)
     int* order = nullptr;      // groups sorted by descending neighbour count
     R2CItem* r2c = nullptr;
     int n_r2c = 0;
@@ -1094,7 +1106,14 @@ static lgf_status build_plan(lgf_plan_s* P, const std::vector<HostPlan>& hp) {
             // reflection-reduced tables where the one-CTA-per-chunk products
             // run (the persistent kernel streams the half table by tensor copies)
             D.oct = P->symmetric_spectra == 1 && kind != kNear && !uses_persist(P, l) && !P->generic;
-            if ((s = get_spectra(P->device, nb, S, h, kind, P->prec, D.kh, D.oct ? 1 : 0)) != LGF_OK) return s;
+            const bool chunks = P->generic && kind != kNear && !uses_persist(P, l);
+            if (chunks) {
+                std::vector<int> mask(size_t(D.n_groups), 0);
+                for (const R2CItem& it : items) mask[size_t(it.dst / 8)] |= 1 << it.dst % 8;
+                if ((s = upload(P, mask, &D.gmask)) != LGF_OK) return s;
+            }
+            const TableForm form = D.oct ? kOct : chunks ? kChunks : kRows;
+            if ((s = get_spectra(P->device, nb, S, h, kind, P->prec, D.kh, form)) != LGF_OK) return s;
             D.pp.tmap = D.kh->has_tmap ? &D.kh->tmap : nullptr;
         }
         if (l >= 1 && !(l == 1 && P->merged && Lmac < 2)) {
@@ -1428,7 +1447,7 @@ static lgf_status solve_impl(lgf_plan_s* P, const T* f, T* u, cudaStream_t st) {
             if (!D.m2l) continue;
             e = timed(P, "mac_interval_l2plus", s2, [&] {
                 if (uses_persist(P, l)) return Lc::mac_persist(D.fh, D.kh->ptr, D.uh, D.pp, P->SI, 0, s2);
-                if (gen) return Gn::mac(D.fh, D.kh->ptr, D.uh, D.gnbr, D.n_groups, P->SI, 0, s2);
+                if (gen) return Gn::mac(D.fh, D.kh->ptr, D.uh, D.gnbr, D.gmask, D.n_groups, P->SI, 0, s2);
                 return Lc::mac_interval(D.fh, D.kh->ptr, D.uh, D.gnbr, D.order, D.n_groups, P->SI, P->interval_kernel,
                                         0, table_map(D), P->err, s2, D.oct ? 1 : 0, P->mac_gpc);
             });
@@ -1485,7 +1504,8 @@ static lgf_status solve_impl(lgf_plan_s* P, const T* f, T* u, cudaStream_t st) {
             const int early = !split && P->ev.empty() ? 1 : 0;
             if (uses_persist(P, 0))
                 return Lc::mac_persist(lev[0].fh, lev[0].kh->ptr, lev[0].uh, lev[0].pp, P->S0, early, st);
-            if (gen) return Gn::mac(lev[0].fh, lev[0].kh->ptr, lev[0].uh, lev[0].gnbr, lev[0].n_groups, P->S0, 1, st);
+            if (gen) return Gn::mac(lev[0].fh, lev[0].kh->ptr, lev[0].uh, lev[0].gnbr, lev[0].gmask, lev[0].n_groups,
+                                    P->S0, 1, st);
             return Lc::mac_interval(lev[0].fh, lev[0].kh->ptr, lev[0].uh, lev[0].gnbr, lev[0].order, lev[0].n_groups,
                                     P->S0, P->interval_kernel == 3 ? 3 : 1, 1, table_map(lev[0]), P->err, st,
                                     lev[0].oct ? 1 : 0, P->mac_gpc);
@@ -1524,7 +1544,7 @@ static lgf_status solve_impl(lgf_plan_s* P, const T* f, T* u, cudaStream_t st) {
             if (e != cudaSuccess) return cuda_fail(e, "interval forward FFT");
             e = timed(P, "mac_interval_l1", s1, [&] {
                 if (uses_persist(P, 1)) return Lc::mac_persist(D.fh, D.kh->ptr, D.uh, D.pp, P->SI, 0, s1);
-                if (gen) return Gn::mac(D.fh, D.kh->ptr, D.uh, D.gnbr, D.n_groups, P->SI, 0, s1);
+                if (gen) return Gn::mac(D.fh, D.kh->ptr, D.uh, D.gnbr, D.gmask, D.n_groups, P->SI, 0, s1);
                 return Lc::mac_interval(D.fh, D.kh->ptr, D.uh, D.gnbr, D.order, D.n_groups, P->SI, P->interval_kernel,
                                         0, table_map(D), P->err, s1, D.oct ? 1 : 0, P->mac_gpc);
             });
