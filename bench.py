@@ -141,7 +141,7 @@ def measure_fma_peaks(lgfm, dev: int):
 
 
 def profiled_traffic(name: str):
-    """DRAM bytes per launch of the dominant kernel from its committed ncu
+    """DRAM bytes per solve of the dominant phase from its committed ncu
     summary (profiles/<kernel>_torus_box_128_fp32.md), or None when there is
     none or the kernel sources changed after that capture."""
     import hashlib
@@ -149,8 +149,8 @@ def profiled_traffic(name: str):
     csrc = os.path.join(ROOT, "paper_1402_6081_gb300", "csrc")
     try:
         text = open(path).read()
-        h = hashlib.sha256(open(os.path.join(csrc, "kernels_impl.cuh"), "rb").read()
-                           + open(os.path.join(csrc, "fft_device.cuh"), "rb").read()).hexdigest()[:16]
+        h = hashlib.sha256(open(os.path.join(csrc, "group_impl.cuh"), "rb").read()
+                           + open(os.path.join(csrc, "group_dft.cuh"), "rb").read()).hexdigest()[:16]
         kv = dict(line.split(": ", 1) for line in text.splitlines() if ": " in line and "_" in line.split(": ")[0]
                   and " " not in line.split(": ")[0])
         if kv.get("kernel_source_sha256_16") != h:
@@ -185,6 +185,22 @@ def interaction_pairs(blocks: np.ndarray, n_levels: int):
                                 n += 1
         out[l] = n
     return out
+
+
+def group_work(blocks: np.ndarray, n_b: int):
+    """Work of the merged level-0/1 products in complex products (8 flop), and
+    its description: one product per frequency of the 4 n_b transform for each
+    pair of neighbouring sibling groups, and the z transforms of the phase (every
+    column forward and back at 5 S log2 S flop)."""
+    groups = set(map(tuple, np.unique(np.asarray(blocks, dtype=np.int64) >> 1, axis=0)))
+    near = [(x, y, z) for x in (-1, 0, 1) for y in (-1, 0, 1) for z in (-1, 0, 1)]
+    pairs = sum((g[0] + d[0], g[1] + d[1], g[2] + d[2]) in groups for g in groups for d in near)
+    S = 4 * n_b
+    cols = (S // 2 + 1) * S
+    lines = 2 * len(groups) * cols
+    return (pairs * cols * S + lines * 5.0 * S * np.log2(S) / 8.0,
+            f"{pairs} neighbour pairs of sibling groups x {cols * S} frequencies"
+            f" + {lines} z transforms of {S} at 5 N log2 N flop")
 
 
 def cpu_oracle_rate(p, spectra=None):
@@ -756,8 +772,7 @@ def main():
             "mac_all_levels": ((pairs[0] + pairs[1]) * nw[0] + sum(a * b for _, a, b in upper),
                                f"({pairs[0]} near + {pairs[1]} level-1 interaction pairs) x {nw[0]} frequencies"
                                + "".join(f" + {a} level-{l} pairs x {b}" for l, a, b in upper)),
-            "mac_level01": ((pairs[0] + pairs[1]) * nw[0],
-                            f"({pairs[0]} near + {pairs[1]} level-1 interaction pairs) x {nw[0]} frequencies"),
+            "mac_level01": group_work(p.blocks, p.n_b),
             "mac_interval_l1": (pairs[1] * nw[1], f"{pairs[1]} interaction pairs x {nw[1]} frequencies")}
     roof = None
     if dom_name in work:
