@@ -1361,7 +1361,9 @@ static lgf_status solve_impl(lgf_plan_s* P, const T* f, T* u, cudaStream_t st) {
     // The grouped phases follow one another on st with nothing in between
     // (events do when launches are timed).  Beside the long levels >= 2 chain
     // of the run-time-size kernels, CTAs that started early and wait hold SMs
-    // that the chain needs (n_b = 24, 144^3: 873 us without, 900 with).
+    // that the chain needs (n_b = 24, 144^3: 873 us without, 900 with, while
+    // Reg, Interp and the products took 554 us; 628 and 625 at today's 250:
+    // nothing lost, nothing to gain).
     const int chain = P->ev.empty() && !(gen && Lm >= 2) ? 1 : 0;
     auto c2r0 = [&](const T* add) -> cudaError_t {
         if (P->grouped)
