@@ -49,6 +49,25 @@ __device__ __forceinline__ cx<T> cmac(cx<T> acc, cx<T> a, cx<T> b) {
     return acc;
 }
 
+// ---- loads of what the preceding kernel wrote ----
+// For kernels that start while their predecessor still runs (programmatic
+// serialization) and wait for it: ordinary loads, ordered behind that wait
+// (both are volatile).  __ldg, or a const __restrict__ pointer, would allow a
+// non-coherent load, which needs data that nobody writes while the kernel
+// lives.
+template <typename T>
+__device__ __forceinline__ cx<T> ld_prev(const cx<T>* p) {
+    cx<T> v;
+    if constexpr (sizeof(T) == 4) asm volatile("ld.global.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
+    else asm volatile("ld.global.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ ulonglong2 ld_prev(const ulonglong2* p) {
+    ulonglong2 v;
+    asm volatile("ld.global.v2.u64 {%0, %1}, [%2];" : "=l"(v.x), "=l"(v.y) : "l"(p));
+    return v;
+}
+
 // ---- twiddle tables ----
 // every transform length S of the supported block sizes (level 0: 2 n_b;
 // levels >= 1: the interval lengths)

@@ -18,6 +18,7 @@ namespace grp {
 
 using dev::cx;
 using dev::czero;
+using dev::ld_prev;
 
 // ---- exp(2 pi i j / n) as constant expressions ----
 // sin and cos of a in [0, pi/4]: 14 terms of the series, below 1e-19

@@ -70,8 +70,19 @@ struct Dim {
 // The kernels of a solve follow one another with programmatic serialization: a
 // kernel may start while its predecessor drains, reads its tables, and waits
 // here before it touches what the predecessor writes or reads (nothing to wait
-// for in a kernel launched the ordinary way).  Four launches of 4 us each: the
-// 32^3 box of 8^3 blocks takes 14.4 us with it, 21.3 without.
+// for in a kernel launched the ordinary way).  Two rules keep that sound:
+//  * What an earlier kernel of the chain writes (xy, spec, images) is read by
+//    ordinary loads (ld_prev) through pointers without __restrict__: the
+//    non-coherent loads that __ldg and const __restrict__ stand for need data
+//    that nobody writes while the kernel lives, and this kernel lives before
+//    its predecessor is done.  Tables of the plan are constant: ld, __ldg.
+//  * A kernel lets its successor start only after its own wait, so at most two
+//    of the chain live at once: none starts beside the last but one, which may
+//    still read a buffer that the one between them rewrites (the images from
+//    band to band, xy in k_gmac).
+// Four launches of 4 us each: the 32^3 box of 8^3 blocks takes 14.3 us with it,
+// 20.5 without (before this file's loads were ordinary ones and the signal
+// stood before the wait: 13.7; larger domains measure the same either way).
 __device__ __forceinline__ void let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void wait_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
@@ -245,7 +256,7 @@ __host__ __device__ constexpr int z_lines() {
     return sizeof(cx<double>) * (32 * size_t(Dim<double, NB>::LINE) + Dim<double, NB>::S) <= 48 * 1024 ? 32 : 16;
 }
 template <int NB>
-__global__ void __launch_bounds__(256) k_gz_fwd(const cx<double>* __restrict__ xy, const cx<double>* __restrict__ tw,
+__global__ void __launch_bounds__(256) k_gz_fwd(const cx<double>* xy, const cx<double>* __restrict__ tw,
                                                 cx<double>* __restrict__ spec, int n_groups) {
     using T = double;
     using D = Dim<T, NB>;
@@ -253,8 +264,8 @@ __global__ void __launch_bounds__(256) k_gz_fwd(const cx<double>* __restrict__ x
     __shared__ cx<T> e[L * LINE];
     __shared__ cx<T> tws[S];
     for (int i = threadIdx.x; i < S; i += 256) tws[i] = ld(tw + i);
-    let_next_start();
     wait_previous();
+    let_next_start();
     __syncthreads();
     const int g = blockIdx.x / PER, c0 = blockIdx.x % PER * L, n = min(L, int(D::NC) - c0);
     for (int t = threadIdx.x; t < n * RB; t += 256) {
@@ -262,7 +273,7 @@ __global__ void __launch_bounds__(256) k_gz_fwd(const cx<double>* __restrict__ x
         const cx<T>* in = xy + D::xy(g, c0 + l);
         cx<T> x[8];
 #pragma unroll
-        for (int a = 0; a < 4; ++a) x[a] = ld(in + D::zoff(RB * a + b));
+        for (int a = 0; a < 4; ++a) x[a] = ld_prev(in + D::zoff(RB * a + b));
 #pragma unroll
         for (int a = 4; a < 8; ++a) x[a] = czero<T>();
         dft<8, -1, 4>(x);
@@ -318,12 +329,12 @@ __device__ __forceinline__ void reach(cx<double> (&acc)[8], cx<double> f, const 
 // rows (ty, tz) of four sources (-1: absent), the next row in flight
 template <int R>
 __device__ __forceinline__ void rows(cx<double> (&acc)[8], cx<double> (&F)[2][4], const cx<double> (&k)[kGroupRows],
-                                     const int4* __restrict__ ids, const cx<double>* __restrict__ spec, int stride) {
+                                     const int4* __restrict__ ids, const cx<double>* spec, int stride) {
     auto load = [&](cx<double>(&n)[4], int4 q) {
-        n[0] = q.x >= 0 ? ld(spec + int64_t(q.x) * stride) : czero<double>();
-        n[1] = q.y >= 0 ? ld(spec + int64_t(q.y) * stride) : czero<double>();
-        n[2] = q.z >= 0 ? ld(spec + int64_t(q.z) * stride) : czero<double>();
-        n[3] = q.w >= 0 ? ld(spec + int64_t(q.w) * stride) : czero<double>();
+        n[0] = q.x >= 0 ? ld_prev(spec + int64_t(q.x) * stride) : czero<double>();
+        n[1] = q.y >= 0 ? ld_prev(spec + int64_t(q.y) * stride) : czero<double>();
+        n[2] = q.z >= 0 ? ld_prev(spec + int64_t(q.z) * stride) : czero<double>();
+        n[3] = q.w >= 0 ? ld_prev(spec + int64_t(q.w) * stride) : czero<double>();
     };
     if constexpr (R == 0) load(F[0], __ldg(ids));
     if constexpr (R < 16) {
@@ -340,7 +351,7 @@ __device__ __forceinline__ void rows(cx<double> (&acc)[8], cx<double> (&F)[2][4]
 
 template <int NB>
 __global__ void __launch_bounds__(Dim<double, NB>::MT)
-    k_gmac(const cx<double>* __restrict__ spec, const cx<double>* __restrict__ kern, const cx<double>* __restrict__ tw,
+    k_gmac(const cx<double>* spec, const cx<double>* __restrict__ kern, const cx<double>* __restrict__ tw,
            cx<double>* __restrict__ xy, const int4* __restrict__ sets, int n_super, int per, int n_groups) {
     using T = double;
     using D = Dim<T, NB>;
@@ -357,8 +368,8 @@ __global__ void __launch_bounds__(Dim<double, NB>::MT)
     cx<T> k[kGroupRows];
 #pragma unroll
     for (int i = 0; i < kGroupRows; ++i) k[i] = ld(kern + int64_t(i) * NW + w);
-    let_next_start();
     wait_previous();
+    let_next_start();
     const int s1 = min(n_super, int(blockIdx.y + 1) * per);
     for (int s = blockIdx.y * per; s < s1; ++s) {
         const int4* ids = sets + int64_t(s) * (kSetInts / 4);
@@ -483,7 +494,7 @@ struct Row { ulonglong2 v[4]; };
 template <int IMG>
 __device__ __forceinline__ Row load_row(const int4 q, const cx<float>* base) {
     // loaded as the 64-bit pairs that are used: a move would wait for the load
-    auto get = [&](int g) { return __ldg(reinterpret_cast<const ulonglong2*>(base + int64_t(g) * IMG)); };
+    auto get = [&](int g) { return ld_prev(reinterpret_cast<const ulonglong2*>(base + int64_t(g) * IMG)); };
     return {{get(q.x), get(q.y), get(q.z), get(q.w)}};
 }
 template <int I, int IMG>
@@ -689,7 +700,7 @@ __device__ __forceinline__ void z_inverse(cx<float>* e, const cx<float>* tws, in
 //   per   sets per unit of a CTA
 template <int NB>
 __global__ void __launch_bounds__(ColDim<NB>::TH, 3)
-    k_gprod(const cx<float>* __restrict__ img, const float4* __restrict__ kern, const cx<float>* __restrict__ tw,
+    k_gprod(const cx<float>* img, const float4* __restrict__ kern, const cx<float>* __restrict__ tw,
             cx<float>* __restrict__ out, const int4* __restrict__ sets, int n_sets, int per, int n_groups,
             int first_col) {
     using C = ColDim<NB>;
@@ -725,8 +736,8 @@ __global__ void __launch_bounds__(ColDim<NB>::TH, 3)
     int s = int(blockIdx.y) * per * C::UNITS + unit;
     const int end = min(n_sets, int(blockIdx.y + 1) * per * C::UNITS);
     int4 next = lane < VEC && s < end ? __ldg(sets + int64_t(s) * VEC + lane) : make_int4(0, 0, 0, 0);
-    let_next_start();
     wait_previous();
+    let_next_start();
     // the record of a set and its first rows come while the set before it is
     // transformed back
     Row ring[kAhead + 1];
@@ -772,7 +783,7 @@ __global__ void __launch_bounds__(ColDim<NB>::TH, 3)
 template <int NB>
 __host__ __device__ constexpr int image_lines() { return ColDim<NB>::LINE <= 72 ? 64 : 32; }
 template <int NB>
-__global__ void __launch_bounds__(256) k_gz_image(const cx<float>* __restrict__ xy, const cx<float>* __restrict__ tw,
+__global__ void __launch_bounds__(256) k_gz_image(const cx<float>* xy, const cx<float>* __restrict__ tw,
                                                   cx<float>* __restrict__ img, int first_col, int band_cols,
                                                   int n_groups) {
     using C = ColDim<NB>;
@@ -782,12 +793,12 @@ __global__ void __launch_bounds__(256) k_gz_image(const cx<float>* __restrict__ 
     __shared__ cx<float> tws[S];
     const int per = (band_cols + L - 1) / L, g = blockIdx.x / per, c0 = blockIdx.x % per * L, n = min(L, band_cols - c0);
     for (int i = threadIdx.x; i < S; i += 256) tws[i] = ld(tw + i);
-    let_next_start();
     wait_previous();
+    let_next_start();
     __syncthreads();
     const cx<float>* in = xy + D::xy(g, first_col + c0);
     z_forward<NB, 2>(e, tws, int(threadIdx.x / 32) * Team<NB>::WARP_LINES, 8 * Team<NB>::WARP_LINES, n,
-                     [&](int l, int z) { return ld(in + l * D::PZ + D::zoff(z)); });
+                     [&](int l, int z) { return ld_prev(in + l * D::PZ + D::zoff(z)); });
     __syncthreads();
     for (int i = threadIdx.x; i < n * (IMG / 2); i += 256) {
         const int l = i / (IMG / 2), v = i % (IMG / 2);
@@ -800,7 +811,7 @@ __global__ void __launch_bounds__(256) k_gz_image(const cx<float>* __restrict__ 
 // Inverse y and x transforms of PZ planes of a group into its blocks.
 template <typename T, int NB>
 __global__ void __launch_bounds__(Dim<T, NB>::TH, sizeof(T) == 4 && NB <= 16 ? 4 : 1)
-    k_gxy_inv(const cx<T>* __restrict__ xy, const int* __restrict__ blk, const int* __restrict__ aux,
+    k_gxy_inv(const cx<T>* xy, const int* __restrict__ blk, const int* __restrict__ aux,
               const cx<T>* __restrict__ tw, T* __restrict__ u, const T* __restrict__ add, int add_n,
               int64_t add_stride) {
     using D = Dim<T, NB>;
@@ -824,7 +835,7 @@ __global__ void __launch_bounds__(Dim<T, NB>::TH, sizeof(T) == 4 && NB <= 16 ? 4
             const cx<T>* q = in + ((k0 + line) * S + c) * PZ;
             cx<T> x[RB];
 #pragma unroll
-            for (int d = 0; d < RB; ++d) x[d] = ld(q + 8 * d * PZ);
+            for (int d = 0; d < RB; ++d) x[d] = ld_prev(q + 8 * d * PZ);
             dft<RB, 1, RB>(x);
 #pragma unroll
             for (int b = 0; b < RB; ++b) p.x(line, c, b) = cmulw(x[b], p.tw[b * c]);
