@@ -951,13 +951,13 @@ __device__ __forceinline__ PairSrc ldg_pair(const PairSrc* p) {
     return {v.x, v.y};
 }
 
+// ordinary loads: k_mac_persist may live while the forward FFT writes fh
 template <int S>
-__device__ __forceinline__ void persist_load(cx<float> (&F)[8], const cx<float>* __restrict__ fh, int src,
-                                             int64_t wc) {
+__device__ __forceinline__ void persist_load(cx<float> (&F)[8], const cx<float>* fh, int src, int64_t wc) {
     constexpr int64_t NWS = (int64_t(S / 2 + 1) * S * S + 31) / 32 * 32;
     const cx<float>* p = fh + int64_t(src) * (8 * NWS) + wc;
 #pragma unroll
-    for (int c = 0; c < 8; ++c) F[c] = ldg_cx(p + c * NWS);
+    for (int c = 0; c < 8; ++c) F[c] = ld_prev(p + c * NWS);
 }
 
 // the 8 x 8 sibling products of one source group; kb: centre row of this lane
@@ -999,7 +999,7 @@ constexpr size_t kPersistSmem = 2 * size_t(kPersistBuf) + 64;
 
 template <int S, int WARPS, bool PACKED>
 __global__ void __launch_bounds__(32 * WARPS, 1)
-    k_mac_persist(const cx<float>* __restrict__ fh, const cx<float>* __restrict__ kh, cx<float>* __restrict__ uh,
+    k_mac_persist(const cx<float>* fh, const cx<float>* __restrict__ kh, cx<float>* __restrict__ uh,
                   const PairSrc* __restrict__ pairs, const int* __restrict__ start, const int* __restrict__ order,
                   const long long* __restrict__ cta_units, int n_groups, int* __restrict__ err,
                   const __grid_constant__ CUtensorMap tmap, int use_tma) {

@@ -17,6 +17,7 @@ CSRC = pathlib.Path(__file__).resolve().parents[1] / "paper_1402_6081_gb300" / "
 READS = {
     "group_impl.cuh": {"k_gz_fwd": "xy", "rows": "spec", "k_gmac": "spec", "load_row": "base", "sources2": "base",
                        "k_gprod": "img", "k_gz_image": "xy", "k_gxy_inv": "xy"},
+    "kernels_impl.cuh": {"persist_load": "fh", "k_mac_persist": "fh"},
 }
 WAIT = re.compile(r"wait_previous\(\)|griddepcontrol\.wait")
 TRIGGER = re.compile(r"let_next_start\(\)|griddepcontrol\.launch_dependents")
