@@ -300,7 +300,7 @@ def batch_run(torch, lgfm, steps: int, warmup: int, flush):
         dt = torch.float64 if prec == lgfm.LGF_FP64 else torch.float32
         bs = lgfm.BatchSolver(specs, prec, use_graph=1, options=opts if prec == lgfm.LGF_FP32 else None)
         bs.set_sources([torch.from_numpy(p.f).to(dt) for p in probs])
-        launches = sum(lgfm.lgf_plan_timings(pl)[1] for pl in bs.plans)
+        launches = sum(lgfm.lgf_plan_kernel_launches(pl) for pl in bs.plans)
         k = steps if prec == lgfm.LGF_FP32 else max(3, steps // 5)
         with torch.cuda.stream(stream):
             for _ in range(warmup):
@@ -710,10 +710,11 @@ def main():
     ms, wall = timed_steps(s32, f32, u32, args.steps, args.warmup)
     clk = clocks.stop()
     total_ms, value = replica_rate(float(sum(ms)), npts, args.steps, world, dist, "cuda")
-    # per-kernel times from a shorter pass with an event pair around every launch
+    # per-phase times from a shorter pass with an event pair around every phase
     k_tr = max(3, min(200, args.steps // 10))
     ms_traced, _ = timed_steps(s32, f32, u32, k_tr, 3, timing_capacity=k_tr * 16)
-    ktimes, per_solve_launches = lgfm.lgf_plan_timings(s32.plan)
+    ktimes, _ = lgfm.lgf_plan_timings(s32.plan)
+    per_solve_launches = lgfm.lgf_plan_kernel_launches(s32.plan)
     lgfm.lgf_plan_set_timing(s32.plan, 0)
 
     # the same kernels once more with every launch on one stream, so the

@@ -408,19 +408,26 @@ lgf_status lgf_solve_host_pipelined(lgf_plan plan, const void *const *f_host, vo
 lgf_status lgf_plan_sync(lgf_plan plan);
 
 /*
- * Per-kernel timing (tracing).  lgf_plan_set_timing(plan, capacity) makes the
- * next solves bracket each kernel launch by a CUDA event pair on the solve's
- * stream, for up to `capacity` launches in total (0 turns it off).
- * lgf_plan_timings waits for those events and returns, per kernel name, the
- * summed elapsed time and the number of launches, then starts a new tally.
+ * Per-phase timing (tracing).  A phase is one step of a solve on one level (a
+ * forward transform, the products, ...): one kernel, or several where the
+ * step's form needs them.  lgf_plan_set_timing(plan, capacity) makes the next
+ * solves bracket each phase by a CUDA event pair on the solve's stream, for up
+ * to `capacity` phases in total (0 turns it off).  lgf_plan_timings waits for
+ * those events and returns, per phase name, the summed elapsed time and the
+ * number of phases, then starts a new tally.
  *   names               max_kernels x 32 chars (NUL-terminated names)
  *   total_ms, count     max_kernels entries
  *   n_kernels           receives the number of distinct names (may exceed max)
- *   launches_per_solve  receives the kernel launches of the last solve (or NULL)
+ *   launches_per_solve  receives the phases of the last solve (or NULL); Reg and
+ *                       Interp with compensated sums in some problems of a
+ *                       plan only count twice
  */
 lgf_status lgf_plan_set_timing(lgf_plan plan, int32_t capacity);
 lgf_status lgf_plan_timings(lgf_plan plan, int32_t max_kernels, int32_t *n_kernels, char *names,
                             double *total_ms, int32_t *count, int32_t *launches_per_solve);
+
+/* Kernels that the plan's last solve launched (0 before the first). */
+lgf_status lgf_plan_kernel_launches(lgf_plan plan, int32_t *launches);
 
 /*
  * lgf_conv_blocks - the FFT convolution of isolated blocks (the special case

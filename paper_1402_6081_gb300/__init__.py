@@ -60,6 +60,7 @@ _SIGS = {
     "lgf_plan_set_timing": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_int32]),
     "lgf_plan_timings": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_int32, ctypes.c_void_p, ctypes.c_void_p,
                                         ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p]),
+    "lgf_plan_kernel_launches": (ctypes.c_int, [ctypes.c_void_p, ctypes.POINTER(ctypes.c_int32)]),
     "lgf_destroy": (ctypes.c_int, [ctypes.c_void_p]),
     "lgf_conv_blocks": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_int64, ctypes.c_int32,
                                        ctypes.c_int32, ctypes.c_void_p]),
@@ -311,8 +312,8 @@ def lgf_plan_set_timing(plan: int, capacity: int) -> None:
 
 
 def lgf_plan_timings(plan: int):
-    """{kernel name: (total_ms, launches)} since the last call, and the kernel
-    launches of the last solve."""
+    """{phase name: (total_ms, count)} since the last call, and the phases of
+    the last solve (lgf_plan_kernel_launches counts its kernels)."""
     mx = 64
     n = ctypes.c_int32()
     names = ctypes.create_string_buffer(32 * mx)
@@ -326,6 +327,13 @@ def lgf_plan_timings(plan: int):
         nm = names.raw[32 * j: 32 * (j + 1)].split(b"\0", 1)[0].decode()
         out[nm] = (tot[j], cnt[j])
     return out, per.value
+
+
+def lgf_plan_kernel_launches(plan: int) -> int:
+    """Kernels that the plan's last solve launched (0 before the first)."""
+    n = ctypes.c_int32()
+    _check(library().lgf_plan_kernel_launches(plan, ctypes.byref(n)), "lgf_plan_kernel_launches")
+    return n.value
 
 
 def lgf_measure_fma_peak(kind: int, reps: int = 5) -> tuple[float, float]:

@@ -492,7 +492,7 @@ cudaError_t axis_pass(const dev::cx<T>* in, const int* in_slots, int64_t in_ws, 
     g_axis<T><<<grid_for(lines, threads), threads, smem, st>>>(in, in_slots, in_ws, out, out_slots, out_ws,
                                                               slot_stride, n, S, nin, nout, n_other, axis_stride,
                                                               other_stride, sign, tw);
-    return cudaGetLastError();
+    return launched();
 }
 
 }  // namespace gen
@@ -515,11 +515,12 @@ cudaError_t Generic<T>::r2c(int S, int n_in, const T* src, int64_t stride, const
     const size_t smem_x = sizeof(C) * S + sizeof(T) * size_t((tile_len - 1) / NX + 2) * n_in;
     gen::g_r2c_x<T><<<unsigned(int64_t(n) * tiles), gen::kThreads, smem_x, st>>>(src, stride, items, tiles, tile_len,
                                                                                  A, nws, S, n_in, tw);
-    cudaError_t e = gen::axis_pass<T>(A, slots, nws, B, nullptr, bws, 2, n, S, n_in, S, n_in, NX, int64_t(S) * NX,
-                                      -1, tw, st);
+    cudaError_t e = launched();
+    if (e == cudaSuccess)
+        e = gen::axis_pass<T>(A, slots, nws, B, nullptr, bws, 2, n, S, n_in, S, n_in, NX, int64_t(S) * NX, -1, tw, st);
     if (e == cudaSuccess)
         e = gen::axis_pass<T>(B, nullptr, bws, A, slots, nws, 2, n, S, n_in, S, S, int64_t(S) * NX, NX, -1, tw, st);
-    return e != cudaSuccess ? e : cudaGetLastError();
+    return e;
 }
 
 template <typename T>
@@ -546,7 +547,7 @@ cudaError_t Generic<T>::c2r(int S, int n_out, const void* spec, const C2RItem* i
     const size_t smem_x = sizeof(C) * (S + size_t((tile_len - 1) / n_out + 2) * NX);
     gen::g_c2r_x<T><<<unsigned(int64_t(n) * tiles), gen::kThreads, smem_x, st>>>(U, items, tiles, tile_len, dst, ds,
                                                                                  add, add_n, as, nws, S, n_out, tw);
-    return cudaGetLastError();
+    return launched();
 }
 
 template <typename T>
@@ -569,7 +570,7 @@ cudaError_t Generic<T>::mac(const void* fh, const void* kh, void* uh, const int*
     gen::g_mac<T><<<grid, block, smem, st>>>(static_cast<const dev::cx<T>*>(fh), static_cast<const dev::cx<T>*>(kh),
                                              static_cast<dev::cx<T>*>(uh), gnbr, mask, n_groups, gpc, include_self, nw,
                                              nws);
-    return cudaGetLastError();
+    return launched();
 }
 
 template <typename T, bool ADJ, bool COMP>
@@ -581,7 +582,7 @@ static cudaError_t launch_planes(const T* src, int in_n, const int* source, cons
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
     if (e != cudaSuccess) return e;
     k<<<unsigned(int64_t(n_items) * slabs), gen::kRiThreads, smem, st>>>(src, in_n, source, slot, slabs, W, NI, slices);
-    return cudaGetLastError();
+    return launched();
 }
 
 template <typename T, bool COMP>
@@ -595,7 +596,7 @@ static cudaError_t launch_reg(int NI, const T* src, int in_n, const int* child_i
     if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem))) != cudaSuccess) return e;
     k<<<unsigned(int64_t(n_parents) * bundles), gen::kRiThreads, smem, st>>>(child_index, parent_slot, in_n, bundles,
                                                                             dst, W, NI, slices);
-    return cudaGetLastError();
+    return launched();
 }
 
 template <typename T, bool COMP>
@@ -609,7 +610,7 @@ static cudaError_t launch_interp(int NI, const int* slot, const int* parent, int
     if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem))) != cudaSuccess) return e;
     k<<<unsigned(int64_t(n_items) * bundles), gen::kRiThreads, smem, st>>>(slot, bundles, u, W, NI, accumulate, block,
                                                                           slices);
-    return cudaGetLastError();
+    return launched();
 }
 
 template <typename T>

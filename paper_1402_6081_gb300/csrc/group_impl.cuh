@@ -921,7 +921,7 @@ static cudaError_t launch_after(void (*kernel)(P...), dim3 grid, int block, size
     at.val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = &at;
     cfg.numAttrs = early ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+    return launched(cudaLaunchKernelEx(&cfg, kernel, P(args)...));
 }
 
 template <typename T, int NB>
@@ -935,7 +935,7 @@ cudaError_t GroupSize<T, NB>::forward(const GroupTables& g, const T* f, void* xy
     auto* p = static_cast<dev::cx<T>*>(xy);
     const auto* tw = static_cast<const dev::cx<T>*>(g.tw);
     k<<<unsigned(g.n_groups * (D::N / D::PZ)), D::TH, smem, st>>>(f, g.blk, tw, p);
-    if ((e = cudaGetLastError()) != cudaSuccess || group_banded<T>()) return e;
+    if ((e = launched()) != cudaSuccess || group_banded<T>()) return e;
     if constexpr (!group_banded<T>()) {
         constexpr int L = grp::z_lines<NB>(), per = (int(D::NC) + L - 1) / L;
         e = launch_after(grp::k_gz_fwd<NB>, dim3(unsigned(g.n_groups * per)), 256, 0, st, early, p, tw,

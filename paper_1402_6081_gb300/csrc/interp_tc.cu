@@ -450,7 +450,7 @@ static cudaError_t launch_interp(const int* slot, const int* parent, int n, floa
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
     if (e != cudaSuccess) return e;
     kern<<<n, kThreads, smem, st>>>(slot, parent, u, up, pack<NI>(W), accumulate, block, err);
-    return cudaGetLastError();
+    return launched();
 }
 
 template <int MODE, int NI>
@@ -464,7 +464,7 @@ static cudaError_t launch_reg(const float* child_src, int child_is_block, const 
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
     if (e != cudaSuccess) return e;
     kern<<<n, kThreads, smem, st>>>(child_src, child_is_block, child_index, parent_slot, dst, pack<NI>(W), err);
-    return cudaGetLastError();
+    return launched();
 }
 
 }  // namespace tc

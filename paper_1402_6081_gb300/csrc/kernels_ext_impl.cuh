@@ -113,7 +113,7 @@ cudaError_t LaunchExt<T>::interp(int n_b, int n_max, const int* slot, const int*
     if (n_b + 1 == NI) {                                                                                      \
         auto kern = comp ? dev::k_interp<T, NI, sizeof(T) == 4, 0> : dev::k_interp<T, NI, false, 0>;            \
         kern<<<n_items, dev::kLineThreads, 0, st>>>(slot, parent, u, up, pack_w<T, NI>(W), accumulate, block); \
-        return cudaGetLastError();                                                                            \
+        return launched();                                                                            \
     }
     LGF_INTERP(7) LGF_INTERP(11) LGF_INTERP(13) LGF_INTERP(15)
 #undef LGF_INTERP

@@ -56,7 +56,7 @@ cudaError_t r2c_cube(int S, int n_in, const CUtensorMap& in_map, const R2CItem* 
         dev::k_r2c_cube<SS, NN><<<g, dev::cube_threads<SS>(), dev::r2c_cube_smem<SS, NN>(), st>>>(in_map, items, \
                                                                                                  n, out, ctr,   \
                                                                                                  err);          \
-        return cudaGetLastError();                                                                               \
+        return launched();                                                                               \
     }
     LGF_R2C_CUBE(32, 16) LGF_R2C_CUBE(16, 8)
 #undef LGF_R2C_CUBE
@@ -72,7 +72,7 @@ cudaError_t c2r_cube(int S, int n_out, const void* spec, const C2RItem* items, i
     if (S == SS && n_out == NN) {                                                                                   \
         dev::k_c2r_cube<SS, NN><<<g, dev::cube_threads<SS>(), dev::c2r_cube_smem<SS, NN>(), st>>>(                 \
             in, items, n, dst, ds, add, add_n, as, ctr, err);                                                      \
-        return cudaGetLastError();                                                                                  \
+        return launched();                                                                                  \
     }
     LGF_C2R_CUBE(32, 16) LGF_C2R_CUBE(16, 8)
 #undef LGF_C2R_CUBE

@@ -2024,7 +2024,7 @@ static cudaError_t launch_r2c(const T* src, int64_t stride, const R2CItem* items
     constexpr int K = dev::fft_items_per_cta<T, S, NIN>();
     k<<<(n + K - 1) / K, dev::fft_threads<T, S, NIN>(), smem, st>>>(src, stride, items,
                                                                      static_cast<dev::cx<T>*>(spec), n);
-    return cudaGetLastError();
+    return launched();
 }
 
 template <typename T, int S, int NOUT>
@@ -2038,7 +2038,7 @@ static cudaError_t launch_c2r(const void* spec, const C2RItem* items, int n, T* 
     constexpr int K = dev::fft_items_per_cta<T, S, NOUT>();
     k<<<(n + K - 1) / K, dev::fft_threads<T, S, NOUT>(), smem, st>>>(static_cast<const dev::cx<T>*>(spec), items,
                                                                       dst, ds, add, add_n, as, n);
-    return cudaGetLastError();
+    return launched();
 }
 
 template <typename T>
@@ -2078,7 +2078,7 @@ cudaError_t Launch<T>::mac_level0(const void* fh, const void* kh, void* uh, cons
     dev::k_mac_level0<T><<<grid, block, 0, st>>>(static_cast<const dev::cx<T>*>(fh),
                                                  static_cast<const dev::cx<T>*>(kh), static_cast<dev::cx<T>*>(uh),
                                                  gnbr, n_groups, NW, NWS);
-    return cudaGetLastError();
+    return launched();
 }
 
 template <typename T, int S>
@@ -2112,7 +2112,7 @@ static cudaError_t launch_mac_interval(const void* fh, const void* kh, void* uh,
         int per = groups_per_cta(2 * dev::kMacPWarps, 1, nchunks);
         dim3 block(32, dev::kMacPWarps), grid((n_groups + per - 1) / per, unsigned(nchunks));
         kern<<<grid, block, smem, st>>>(f, k, u, gnbr, order, n_groups, per, include_self);
-        return cudaGetLastError();
+        return launched();
     }
     // FP32 outside variant 1: packed two-wide FMAs, 8 warps of up to 128
     // registers (two CTAs per SM); variant 1 and FP64: one FMA per real
@@ -2133,7 +2133,7 @@ static cudaError_t launch_mac_interval(const void* fh, const void* kh, void* uh,
     if (tmap) map = *tmap;
     kern<<<grid, block, smem, st>>>(f, k, u, gnbr, order, n_groups, per, include_self, map, tmap && !oct ? 1 : 0, err,
                                     oct);
-    return cudaGetLastError();
+    return launched();
 }
 
 template <typename T>
@@ -2177,9 +2177,10 @@ static cudaError_t launch_mac_persist(const void* fh, const void* kh, void* uh, 
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = early ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, kern, static_cast<const dev::cx<float>*>(fh),
-                              static_cast<const dev::cx<float>*>(kh), static_cast<dev::cx<float>*>(uh), pp.pairs,
-                              pp.start, pp.order, pp.cta_units, pp.n_groups, pp.err, map, pp.tmap ? 1 : 0);
+    return launched(cudaLaunchKernelEx(&cfg, kern, static_cast<const dev::cx<float>*>(fh),
+                                       static_cast<const dev::cx<float>*>(kh), static_cast<dev::cx<float>*>(uh),
+                                       pp.pairs, pp.start, pp.order, pp.cta_units, pp.n_groups, pp.err, map,
+                                       pp.tmap ? 1 : 0));
 }
 
 template <int S>
@@ -2221,7 +2222,7 @@ static cudaError_t launch_reg(const T* child_src, int child_is_block, const int*
     if constexpr (sizeof(T) == 8) {
         dev::k_reg<T, NI, NMAX><<<n_parents, dev::kLineThreads, 0, st>>>(child_src, child_is_block, child_index,
                                                                         parent_slot, dst, pack_w<T, NI>(W));
-        return cudaGetLastError();
+        return launched();
     } else {
         constexpr size_t smem = dev::reg_wide_smem<T, NI>();
         auto kern = comp ? dev::k_reg_wide<T, NI, true, NMAX> : dev::k_reg_wide<T, NI, false, NMAX>;
@@ -2229,7 +2230,7 @@ static cudaError_t launch_reg(const T* child_src, int child_is_block, const int*
         if (e != cudaSuccess) return e;
         kern<<<n_parents, dev::kRegThreads, smem, st>>>(child_src, child_is_block, child_index, parent_slot, dst,
                                                         pack_w<T, NI>(W));
-        return cudaGetLastError();
+        return launched();
     }
 }
 
@@ -2260,7 +2261,7 @@ cudaError_t Launch<T>::interp(int n_b, int n_max, const int* slot, const int* pa
     if (n_b + 1 == NI && nm == NM) {                                                                          \
         auto kern = comp ? dev::k_interp<T, NI, sizeof(T) == 4, NM> : dev::k_interp<T, NI, false, NM>;          \
         kern<<<n_items, dev::kLineThreads, 0, st>>>(slot, parent, u, up, pack_w<T, NI>(W), accumulate, block); \
-        return cudaGetLastError();                                                                            \
+        return launched();                                                                            \
     }
     LGF_INTERP(5, 0) LGF_INTERP(9, 0) LGF_INTERP(9, 7) LGF_INTERP(9, 9) LGF_INTERP(17, 0) LGF_INTERP(17, 7)
     LGF_INTERP(17, 9)

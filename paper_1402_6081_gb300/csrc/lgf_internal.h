@@ -31,6 +31,15 @@ void fft_inplace(std::complex<double>* x, int n, int stride, int sign);
 void fft_lines(std::complex<double>* base, int n, int stride, int count, int64_t line_stride,
                int sign);
 
+// Kernels that the calling thread has launched: the launch helpers end with
+// launched(), so that a solve can tell how many are its own.
+inline thread_local int64_t t_launches = 0;
+inline cudaError_t launched(cudaError_t e) {
+    ++t_launches;
+    return e;
+}
+inline cudaError_t launched() { return launched(cudaGetLastError()); }
+
 // ---- kernel spectra (plan.cpp) ----
 // Spectrum (NW values, w = (kz*S + ky)*NX + kx, scaled by 1/S^3) of the kernel
 // vector k(m) = G(h (m - d n_b)), |m_a| <= n - 1, placed at m mod S; tab is the

@@ -487,7 +487,9 @@ struct lgf_plan_s {
     std::vector<cudaEvent_t> ev;           // 2 * capacity events
     std::vector<const char*> ev_name;      // kernel name per recorded pair
     int ev_used = 0;
-    int launches_last = 0;                 // kernels launched by the last solve
+    int launches_last = 0;                 // phases of the last solve (timed brackets)
+    int64_t launch_base = 0;               // t_launches when the last solve began
+    int kernels_last = 0;                  // kernels launched by the last solve
     // the level-1 chain and the level >= 2 chain run on their own streams,
     // forked from and joined into the caller's stream
     cudaStream_t aux[2] = {nullptr, nullptr};
@@ -1281,7 +1283,7 @@ static lgf_status build_plan(lgf_plan_s* P, const std::vector<HostPlan>& hp) {
 // A level's kernel table as a tensor map, when TMA loads are available for it
 static const CUtensorMap* table_map(const DevLevel& D) { return D.kh && D.kh->has_tmap ? &D.kh->tmap : nullptr; }
 
-// Runs one launch; with timing enabled, brackets it by an event pair on `st`.
+// Runs one phase; with timing enabled, brackets it by an event pair on `st`.
 template <typename F>
 static cudaError_t timed(lgf_plan_s* P, const char* name, cudaStream_t st, F&& launch) {
     ++P->launches_last;
@@ -1291,6 +1293,7 @@ static cudaError_t timed(lgf_plan_s* P, const char* name, cudaStream_t st, F&& l
     nvtxRangePushA(name);   // host-side range per launch, seen by profilers
     cudaError_t e = launch();
     nvtxRangePop();
+    P->kernels_last = int(t_launches - P->launch_base);
     if (rec) {
         cudaEventRecord(P->ev[size_t(2 * k + 1)], st);
         P->ev_name[size_t(k)] = name;
@@ -1303,6 +1306,8 @@ template <typename T>
 static lgf_status solve_impl(lgf_plan_s* P, const T* f, T* u, cudaStream_t st) {
     using Lc = Launch<T>;
     P->launches_last = 0;
+    P->launch_base = t_launches;
+    P->kernels_last = 0;
     const int nb = P->n_b, nI = P->n_I;
     const int64_t n3 = int64_t(nI) * nI * nI, b3 = int64_t(nb) * nb * nb;
     auto& lev = P->lev;
@@ -1992,6 +1997,12 @@ lgf_status lgf_plan_timings(lgf_plan plan, int32_t max_kernels, int32_t* n_kerne
     }
     if (launches_per_solve) *launches_per_solve = plan->launches_last;
     plan->ev_used = 0;
+    return ok();
+}
+
+lgf_status lgf_plan_kernel_launches(lgf_plan plan, int32_t* launches) {
+    if (!plan || !launches) return fail(LGF_ERR_INVALID_ARG, "lgf_plan_kernel_launches: NULL argument");
+    *launches = plan->kernels_last;
     return ok();
 }
 
