@@ -458,9 +458,13 @@ struct lgf_plan_s {
     // first n_b nodes of a level-1 interval: their products are summed into
     // one spectrum per block (one inverse FFT, no level-1 transforms)
     bool merged = true;
-    // merged levels 0 and 1 by whole sibling groups (group.h)
+    // merged levels 0 and 1 by whole sibling groups (group.h), for the
+    // problems that grouping pays for; level 0 of lev holds the others
     bool grouped = false;
     lgf::GroupTables grp;
+    void* gxy = nullptr;    // lines of the x, y transforms; FP64: also back
+    void* gspec = nullptr;  // FP64: spectra; FP32: the lines back
+    std::shared_ptr<lgf::SpecEntry> gkh;
     std::vector<lgf::DevLevel> lev;
     std::vector<int64_t> pairs, intervals, groups;   // per level, for lgf_plan_get_stats
     void* W = nullptr;                  // device copy (unused by the kernels, kept for tools)
@@ -512,6 +516,7 @@ struct lgf_plan_s {
         // cudaFree below (lev.clear()): let the plan's last solve finish first
         bool last_owner = false;
         for (const auto& D : lev) last_owner = last_owner || (D.kh && D.kh.use_count() == 1);
+        last_owner = last_owner || (gkh && gkh.use_count() == 1);
         if (last_owner && done_ev) cudaEventSynchronize(done_ev);
         if (mem_st) {
             if (done_ev) cudaStreamWaitEvent(mem_st, done_ev, 0);
@@ -532,6 +537,7 @@ struct lgf_plan_s {
         for (cudaEvent_t j : join)
             if (j) cudaEventDestroy(j);
         lev.clear();
+        gkh.reset();
         cudaSetDevice(cur);
     }
 };
@@ -626,6 +632,7 @@ struct HostPlan {
     int64_t n_blocks = 0;
     std::vector<HostLevel> lev;                // levels 0..Lmac
     std::vector<int64_t> pairs, intervals, groups;   // levels 0..L
+    bool by_group = false;                     // levels 0 and 1 by whole sibling groups
 };
 
 // Bounds checks of the tables a plan hands to its kernels, on the host before
@@ -891,16 +898,60 @@ static lgf_status build_host(const int32_t* ijk, int64_t NB, int L, HostPlan& H)
     return ok();
 }
 
+// Whether levels 0 and 1 run by whole sibling groups.  That form transforms a
+// group whole, however few of its blocks are there, and takes a set of 2^3
+// target groups at a time, however few of those: where blocks are scattered
+// the blocks' own transforms of 2 n_b are less work.  Counted per problem and
+// summed: sets beyond the first (one set is bound by latency in either form),
+// groups, pairs of neighbouring groups, the blocks those pairs read (where
+// products skip absent sources), blocks.  The weights fit the difference of
+// both forms' solve times over 27 block lists per n_b and precision (boxes,
+// balls, shells, sheets, lines, isolated groups, random blocks and groups, 60 to
+// 6000 blocks); the side taken is the faster one, or within 10%, for 697 of
+// the 702 (the others take groups in FP64: a single group at n_b = 10 and 12,
+// 1.3 to 1.9 times its own form's time, and lines at n_b = 14, 1.13).  us,
+// grouped / blocks' own: 16^3 blocks, FP32, a 5^3 box of full groups 854 / 1045, 1% of a box's
+// blocks 1983 / 1444; FP64 9631 / 23237 and 36536 / 31556; 18^3 FP64 1% 45453
+// / 21902.  Sums of equal problems scale alike, so a problem folded with copies
+// of itself takes the form that it takes alone.
+static bool grouping_pays(int prec, int n_b, const HostPlan* hp, size_t n) {
+    int64_t sets = 0, groups = 0, pairs = 0, sources = 0, blocks = 0;
+    for (size_t p = 0; p < n; ++p) {
+        const HostPlan& H = hp[p];
+        const HostLevel& T = H.lev[0];
+        std::unordered_set<uint64_t> s;
+        for (const I3& g : T.gpos) s.insert(pack(parent_of(g)));
+        std::vector<int> members(size_t(T.n_groups), 0);
+        for (int slot : T.iv_slot) ++members[size_t(slot / 8)];
+        for (int g : T.gn)
+            if (g >= 0) {
+                ++pairs;
+                sources += members[size_t(g)];
+            }
+        sets += int64_t(s.size()) - 1;
+        groups += T.n_groups;
+        blocks += H.n_blocks;
+    }
+    if (prec == LGF_FP32) {
+        if (n_b <= 16) return 128 * sets <= 4 * pairs + 3 * blocks;
+        // transforms of the blocks in shared memory, or an axis per launch
+        return n_b <= 20 ? 64 * sets <= pairs + blocks : 28 * sets + 4 * groups <= pairs + 4 * blocks;
+    }
+    return n_b <= 16 ? 12 * sets <= 2 * pairs + blocks : 200 * sets + 32 * groups <= sources + 32 * blocks;
+}
+
 // Tables and buffers of the grouped level-0/1 convolution: the children's
 // blocks and level-1 slots of every group, and the sets of 2^3 target groups
 // with the 4^3 groups around them (n_groups1: groups at level 1).  A set never spans two problems, and its
 // place depends on the group indices alone, so a problem's sums run in the
-// same order whatever other problems share the plan.
+// same order whatever other problems share the plan.  Only the problems that go
+// by groups take part; n_groups: theirs at level 0.
 static lgf_status build_group(lgf_plan_s* P, const std::vector<HostPlan>& hp, const std::vector<int>& boff,
-                              const std::vector<std::vector<int>>& goff, int n_groups1, DevLevel& D, size_t cplx) {
-    std::vector<int> blk(size_t(D.n_groups) * 8, -1), aux(size_t(D.n_groups) * 8, -1), sup;
+                              const std::vector<std::vector<int>>& goff, int n_groups, int n_groups1, size_t cplx) {
+    std::vector<int> blk(size_t(n_groups) * 8, -1), aux(size_t(n_groups) * 8, -1), sup;
     for (size_t p = 0; p < hp.size(); ++p) {
         const HostPlan& H = hp[p];
+        if (!H.by_group) continue;
         const HostLevel& T = H.lev[0];
         const int g0 = goff[0][p];
         for (int64_t b = 0; b < H.n_blocks; ++b) {
@@ -927,12 +978,12 @@ static lgf_status build_group(lgf_plan_s* P, const std::vector<HostPlan>& hp, co
     lgf_status s;
     if ((s = check_range("group block", blk, -1, P->n_blocks)) != LGF_OK) return s;
     if ((s = check_range("group level-1 slot", aux, -1, 8LL * n_groups1)) != LGF_OK) return s;
-    if ((s = check_range("group set", sup, -1, D.n_groups)) != LGF_OK) return s;
+    if ((s = check_range("group set", sup, -1, n_groups)) != LGF_OK) return s;
     const int S = 4 * P->n_b;
-    const size_t column_set = size_t(D.n_groups) * size_t(group_columns(P->n_b)) * cplx;
+    const size_t column_set = size_t(n_groups) * size_t(group_columns(P->n_b)) * cplx;
     const bool f32 = P->prec == LGF_FP32;
-    if ((s = dalloc(P, column_set * size_t(f32 ? S / 2 : S), &D.fh, false)) != LGF_OK) return s;
-    if ((s = dalloc(P, column_set * size_t(S / 2), &D.uh, false)) != LGF_OK) return s;
+    if ((s = dalloc(P, column_set * size_t(f32 ? S / 2 : S), &P->gspec, false)) != LGF_OK) return s;
+    if ((s = dalloc(P, column_set * size_t(S / 2), &P->gxy, false)) != LGF_OK) return s;
     int *dblk = nullptr, *daux = nullptr, *dsets = nullptr;
     if ((s = upload(P, blk, &dblk)) != LGF_OK) return s;
     if ((s = upload(P, aux, &daux)) != LGF_OK) return s;
@@ -942,13 +993,13 @@ static lgf_status build_group(lgf_plan_s* P, const std::vector<HostPlan>& hp, co
         int rows = 0;
         for (size_t k = 0; k < 64; ++k) {
             if (sup[i + k] >= 0) rows |= 1 << (k / 4);
-            sets.push_back(sup[i + k] >= 0 || !f32 ? sup[i + k] : D.n_groups);
+            sets.push_back(sup[i + k] >= 0 || !f32 ? sup[i + k] : n_groups);
         }
         sets.insert(sets.end(), sup.begin() + long(i) + 64, sup.begin() + long(i) + 72);
         sets.insert(sets.end(), {rows, 0, 0, 0});
     }
     if ((s = upload(P, sets, &dsets)) != LGF_OK) return s;
-    P->grp.n_groups = D.n_groups;
+    P->grp.n_groups = n_groups;
     P->grp.n_super = int(sup.size() / 72);
     P->grp.blk = dblk;
     P->grp.aux = daux;
@@ -956,7 +1007,7 @@ static lgf_status build_group(lgf_plan_s* P, const std::vector<HostPlan>& hp, co
     if (f32) {
         // bands of whole column sets whose images fill about 48 MB of L2
         const GroupShape gs = group_shape(P->n_b);
-        const int64_t column = int64_t(D.n_groups + 1) * gs.image * int64_t(cplx);
+        const int64_t column = int64_t(n_groups + 1) * gs.image * int64_t(cplx);
         const int64_t nc = group_columns(P->n_b), most = std::max<int64_t>(32, int64_t(48 << 20) / column);
         const int64_t bands = (nc + most - 1) / most;
         P->grp.band_cols = int(std::min((nc / bands + 31) / 32 * 32, nc));
@@ -977,7 +1028,7 @@ static lgf_status build_group(lgf_plan_s* P, const std::vector<HostPlan>& hp, co
         if ((s = upload(P, std::vector<float>(t.begin(), t.end()), &d)) != LGF_OK) return s;
         P->grp.tw = d;
     }
-    return get_spectra(P->device, P->n_b, S, 1, kGroup, P->prec, D.kh);
+    return get_spectra(P->device, P->n_b, S, 1, kGroup, P->prec, P->gkh);
 }
 
 // Concatenates the problems' tables level by level and builds the device
@@ -1009,11 +1060,13 @@ static lgf_status build_plan(lgf_plan_s* P, const std::vector<HostPlan>& hp) {
     for (size_t p = 1; p < np; ++p) boff[p] = boff[p - 1] + int(hp[p - 1].n_blocks);
     std::vector<std::vector<int>> goff(size_t(Lmac) + 1, std::vector<int>(np, -1));
     std::vector<int> ngroups(size_t(Lmac) + 1, 0);
+    int n_grouped = 0;   // level-0 groups of the problems that go by groups, counted apart
     for (int l = 0; l <= Lmac; ++l)
         for (size_t p = 0; p < np; ++p)
             if (l <= hp[p].Lmac) {
-                goff[size_t(l)][p] = ngroups[size_t(l)];
-                ngroups[size_t(l)] += hp[p].lev[size_t(l)].n_groups;
+                int& n = l == 0 && hp[p].by_group ? n_grouped : ngroups[size_t(l)];
+                goff[size_t(l)][p] = n;
+                n += hp[p].lev[size_t(l)].n_groups;
             }
     const size_t elem = P->prec == LGF_FP64 ? sizeof(double) : sizeof(float);
     const size_t cplx = 2 * elem;
@@ -1059,9 +1112,10 @@ static lgf_status build_plan(lgf_plan_s* P, const std::vector<HostPlan>& hp) {
         D.m2l = (l == 0) || (any && !(l == 1 && P->merged));
         const size_t slots = size_t(D.n_groups) * 8;
         lgf_status s;
-        if (l == 0 && P->grouped) {
-            if ((s = build_group(P, hp, boff, goff, Lmac >= 1 ? ngroups[1] : 0, D, cplx)) != LGF_OK) return s;
-        } else if (D.m2l) {
+        if (l == 0 && P->grouped &&
+            (s = build_group(P, hp, boff, goff, n_grouped, Lmac >= 1 ? ngroups[1] : 0, cplx)) != LGF_OK)
+            return s;
+        if (D.m2l && D.n_groups > 0) {
             const int S = l == 0 ? P->S0 : P->SI;
             const size_t NWS = size_t(nws_of(S));
             if ((s = dalloc(P, slots * NWS * cplx, &D.fh, true)) != LGF_OK) return s;
@@ -1069,7 +1123,7 @@ static lgf_status build_plan(lgf_plan_s* P, const std::vector<HostPlan>& hp) {
             std::vector<int> gn;
             std::vector<R2CItem> items;
             for (size_t p = 0; p < np; ++p) {
-                if (go[p] < 0) continue;
+                if (go[p] < 0 || (l == 0 && hp[p].by_group)) continue;
                 const HostLevel& T = hp[p].lev[size_t(l)];
                 for (int v : T.gn) gn.push_back(v >= 0 ? v + go[p] : -1);
                 for (const R2CItem& it : T.r2c)
@@ -1178,10 +1232,11 @@ static lgf_status build_plan(lgf_plan_s* P, const std::vector<HostPlan>& hp) {
     }
     // level-0 output items: block b from its level-0 slot, plus its level-1
     // field (same slot number within the problem, level-1 group offset)
-    if (!P->grouped) {
+    {
         std::vector<C2RItem> items;
         for (size_t p = 0; p < np; ++p) {
             const HostPlan& H = hp[p];
+            if (H.by_group) continue;
             const bool has_ut1 = P->merged ? H.Lmac >= 2 : H.Lmac >= 1;
             const std::vector<int>& s0 = H.lev[0].iv_slot;
             for (int64_t b = 0; b < H.n_blocks; ++b)
@@ -1260,7 +1315,7 @@ static lgf_status build_plan(lgf_plan_s* P, const std::vector<HostPlan>& hp) {
         for (int l = 0; l <= Lmac; ++l) {
             DevLevel& D = P->lev[size_t(l)];
             const int S = l == 0 ? P->S0 : P->SI;
-            if (l == 0 && P->grouped) continue;
+            if (D.n_groups == 0) continue;
             if (P->prec == LGF_FP32 && fft_large_supported(S, nb) && (l == 0 || fft_large_supported(S, nI)))
                 continue;
             const size_t items = size_t(std::max({D.n_r2c, D.n_c2r, l == 0 ? P->n_out : 0}));
@@ -1369,11 +1424,16 @@ static lgf_status solve_impl(lgf_plan_s* P, const T* f, T* u, cudaStream_t st) {
     // that the chain needs (n_b = 24, 144^3: 873 us without, 900 with, while
     // Reg, Interp and the products took 554 us; 628 and 625 at today's 250:
     // nothing lost, nothing to gain).
-    const int chain = P->ev.empty() && !(gen && Lm >= 2) ? 1 : 0;
+    // Problems of the blocks' own form in the plan launch in between: no early
+    // starts there.
+    const bool own = lev[0].n_groups > 0;
+    const int chain = P->ev.empty() && !own && !(gen && Lm >= 2) ? 1 : 0;
     auto c2r0 = [&](const T* add) -> cudaError_t {
-        if (P->grouped)
-            return Group<T>::inverse(nb, P->grp, group_banded<T>() ? lev[0].fh : lev[0].uh, u, add, nI, n3,
-                                     Lm < 2 ? chain : 0, st);
+        if (P->grouped) {
+            const cudaError_t r = Group<T>::inverse(nb, P->grp, group_banded<T>() ? P->gspec : P->gxy, u, add, nI, n3,
+                                                    Lm < 2 ? chain : 0, st);
+            if (r != cudaSuccess || !own) return r;
+        }
         if constexpr (std::is_same_v<T, float>)
             if (P->fft_kernel == 2)
                 return c2r_cube(P->S0, nb, lev[0].uh, P->out_items, P->n_out, u, b3, add, nI, n3, P->cube_grid[1],
@@ -1488,7 +1548,10 @@ static lgf_status solve_impl(lgf_plan_s* P, const T* f, T* u, cudaStream_t st) {
     }
     // ---- level 0 on the caller's stream: forward FFT, near-field products
     e = timed(P, "r2c_level0", st, [&] {
-        if (P->grouped) return Group<T>::forward(nb, P->grp, f, lev[0].uh, lev[0].fh, chain, st);
+        if (P->grouped) {
+            const cudaError_t r = Group<T>::forward(nb, P->grp, f, P->gxy, P->gspec, chain, st);
+            if (r != cudaSuccess || !own) return r;
+        }
         if constexpr (std::is_same_v<T, float>)
             if (P->fft_kernel == 2) {
                 if (P->in_map_src != f)
@@ -1503,9 +1566,11 @@ static lgf_status solve_impl(lgf_plan_s* P, const T* f, T* u, cudaStream_t st) {
     if (split) LGF_CUDA(wait(st, 1));
     if (P->merged) {
         e = timed(P, "mac_level01", st, [&] {
-            if (P->grouped)
-                return Group<T>::products(nb, P->grp, group_banded<T>() ? lev[0].uh : lev[0].fh, lev[0].kh->ptr,
-                                          group_banded<T>() ? lev[0].fh : lev[0].uh, chain, st);
+            if (P->grouped) {
+                const cudaError_t r = Group<T>::products(nb, P->grp, group_banded<T>() ? P->gxy : P->gspec, P->gkh->ptr,
+                                                         group_banded<T>() ? P->gspec : P->gxy, chain, st);
+                if (r != cudaSuccess || !own) return r;
+            }
             // directly behind the forward FFT on st (no event between them):
             // launched early, it stages its first coefficient chunks meanwhile
             const int early = !split && P->ev.empty() ? 1 : 0;
@@ -1718,9 +1783,6 @@ static lgf_status create_plan(const int32_t* block_ijk, const int64_t* offsets, 
             P->nmax_lv[size_t(k) + 2] = o + 1;
         }
     }
-    // The grouped form unless the options ask for a product or transform form
-    // of the blocks' own spectra.
-    P->grouped = P->merged && P->interval_kernel == 0 && P->fft_kernel != 2 && group_supported(n_b);
     lgf_status s = ensure_twiddles(P->device, precision);
     if (s != LGF_OK) return s;
     std::vector<HostPlan> hp(static_cast<size_t>(n_problems));
@@ -1729,6 +1791,17 @@ static lgf_status create_plan(const int32_t* block_ijk, const int64_t* offsets, 
         if (s != LGF_OK) {
             if (n_problems > 1) fail(s, "problem " + std::to_string(p) + ": " + g_err);
             return s;
+        }
+    }
+    // The grouped form where it pays, unless the options ask for a product or
+    // transform form of the blocks' own spectra.  FP64: decided per problem, so
+    // that each keeps the bits that a plan of it alone computes; FP32, whose
+    // product forms go by the plan's group counts anyway, once for the plan.
+    if (P->merged && P->interval_kernel == 0 && P->fft_kernel != 2 && group_supported(n_b)) {
+        const bool all = precision == LGF_FP32 && grouping_pays(precision, n_b, hp.data(), hp.size());
+        for (HostPlan& H : hp) {
+            H.by_group = precision == LGF_FP32 ? all : grouping_pays(precision, n_b, &H, 1);
+            P->grouped = P->grouped || H.by_group;
         }
     }
     if (P->free_sms == 0) {
@@ -1802,6 +1875,7 @@ lgf_status lgf_plan_workspace_bytes(lgf_plan plan, size_t* bytes) {
     size_t b = plan->bytes;
     for (auto& D : plan->lev)
         if (D.kh) b += D.kh->bytes;
+    if (plan->gkh) b += plan->gkh->bytes;
     *bytes = b;
     return ok();
 }
