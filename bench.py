@@ -577,7 +577,7 @@ def serve_run(torch, lgfm, n_requests: int = 2200, n_warm: int = 200, precisions
     out["config"] = {"workload": "serve_poisson200", "requests_timed": n_requests - n_warm, "warmup": n_warm,
                      "shapes": len(shapes), "hbm_budget_gb": 120, "streams": 16,
                      "latency": "arrival to result in pinned host memory",
-                     "large_requests": "more than 2^25 points: default-priority stream, plan leaves 32 SMs free "
+                     "large_requests": "more than 2^25 points: all of the plan at the default priority "
                                        "(others on high-priority streams)"}
     return out
 

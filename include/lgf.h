@@ -188,11 +188,16 @@ lgf_status lgf_plan_create(const int32_t *block_ijk, int64_t n_blocks, int32_t n
  *                      the parent neighbourhood (343 kernel offsets) and one
  *                      inverse FFT.  1: separate level-1 transforms of length
  *                      S_I, as the level interactions of Sec. 3.1 are listed.
- *   free_sms           schedule of the persistent level-0 products (interval_kernel
- *                      4 and 5; no effect on the grouped form): -1 = they take every SM and levels >= 2 run
- *                      before and after them; k > 0 = they take all but k SMs
- *                      and levels >= 2 run beside them on the rest; 0 = the
- *                      library's choice
+ *   free_sms           schedule of the levels >= 2 beside the level-0 products.
+ *                      Persistent products (interval_kernel 4 and 5, and
+ *                      default plans whose blocks keep their own transforms):
+ *                      -1 = they take every SM and levels >= 2 run before and
+ *                      after them; k > 0 = they take all but k SMs and levels
+ *                      >= 2 run beside them on the rest.  The grouped form
+ *                      holds no SM for long: levels >= 2 run beside it at the
+ *                      highest stream priority, or with k > 0, whatever k, at
+ *                      the default priority, so that they do not go before the
+ *                      work of other streams.  0 = the library's choice
  *   fft_kernel         level-0 forward and inverse FFTs: 1 = one CTA per block
  *                      (the input and output cubes through per-thread loads
  *                      and stores); 2 = persistent, one CTA per SM taking

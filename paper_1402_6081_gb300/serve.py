@@ -296,12 +296,12 @@ class GpuServer:
     folded result has the bits of the same request solved alone.
 
     Large requests (more than big_points points) run on a stream of the
-    default priority and their plans leave big_free_sms SMs to everything
-    else (option free_sms, unless the tuned options set it): the persistent
-    products of a large solve would otherwise hold every SM for milliseconds,
-    and the requests that arrive meanwhile (their streams at high priority)
-    would wait for them.  The large solve itself takes longer; the others see
-    the free SMs."""
+    default priority, the others on high-priority streams, and large plans
+    leave room to everything else (option free_sms = big_free_sms, unless the
+    tuned options set it): the levels >= 2 of a grouped plan run at the default
+    priority too instead of before every other stream's work, and persistent
+    products, where a plan has them, leave that many SMs free instead of holding
+    every SM for milliseconds."""
 
     def __init__(self, precision: int, problems: dict, budget_bytes: float = 120e9, n_streams: int = 16,
                  tuned_options=None, source=None, keep_results: bool = False, background_plans: bool = True,
