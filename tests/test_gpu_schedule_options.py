@@ -66,3 +66,30 @@ def test_grouped_plan_that_leaves_room_takes_no_precedence():
         assert (min(pr) < 0) == first, (free, pr)
         s.close()
     assert torch.equal(us[0], us[1]) and torch.equal(us[0], us[2])   # a schedule only
+
+
+_refs = {}
+
+
+@pytest.mark.parametrize("n_b", [6, 12, 16, 18])
+@pytest.mark.parametrize("opts", [{"free_sms": -1}, {"free_sms": 24}, {"free_sms": 24, "single_stream": 1}])
+def test_persistent_level0_schedules(n_b, opts):
+    # before and after the products (-1), and beside them; FP32, against the
+    # grouped form, each within 1e-5 of the exact method
+    nb = 6 if n_b <= 12 else 5
+    p = W.torus_box(seed=n_b, nb=nb, n_b=n_b, radius=0.3 * nb * n_b, sigma=0.06 * nb * n_b, n_levels=3)
+    f = torch.from_numpy(p.f).float().cuda()
+
+    def solve(**o):
+        s = lgfm.Solver(p.blocks, p.n_b, p.n_levels, min(8, n_b), lgfm.LGF_FP32, **o)
+        st, u = s.stats(), s(f)
+        lgfm.lgf_plan_sync(s.plan)
+        s.close()
+        return st, u.double()
+
+    if n_b not in _refs:
+        _refs[n_b] = solve()
+    st, u = solve(interval_kernel=5, **opts)
+    ref_st, ref = _refs[n_b]
+    assert st["persistent_ctas"] > 0 and st["top_product_level"] >= 2 and ref_st["persistent_ctas"] == 0
+    assert float((u - ref).abs().max()) <= 2e-5 * float(ref.abs().max())
