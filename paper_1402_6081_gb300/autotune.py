@@ -10,8 +10,8 @@ reflection-reduced ones) and the interaction-list chunk (sibling groups per
 CTA of the one-CTA-per-chunk products).  The search is coordinate-wise: from
 the library's defaults, each dimension in turn is set to each of its values
 with the others held at the best so far.  Results are cached per (GPU name,
-n_b, precision, levels, block-count bucket) in a JSON file ($LGF_TUNE_CACHE,
-default ~/.cache/paper_1402_6081_gb300/autotune.json).
+n_b, precision, levels, block-count bucket, generation of the forms) in a JSON
+file ($LGF_TUNE_CACHE, default ~/.cache/paper_1402_6081_gb300/autotune.json).
 """
 from __future__ import annotations
 
@@ -26,6 +26,13 @@ import numpy as np
 from . import LGF_FP32
 
 _LOCK = threading.Lock()
+
+# Generation of the forms that a default plan picks, part of the cache key:
+# choices made against other defaults are searched again.  1 (keys without
+# it): the blocks' own transforms at levels 0 and 1; 2: sibling groups there,
+# 1.6 times faster at 128^3 than the interval_kernel or fft_kernel = 2 that a
+# search of generation 1 may have stored.
+FORMS = 2
 
 # Values per dimension (0 = the library's choice).  interval_kernel: 1 = one
 # CTA per frequency chunk, 3 = paired groups; free_sms: SMs left to levels >= 2
@@ -75,7 +82,7 @@ def _key(n_b, precision, n_levels, n_blocks) -> str:
     import torch
     dev = torch.cuda.get_device_name(torch.cuda.current_device())
     bucket = 1 << max(0, int(math.ceil(math.log2(max(1, n_blocks)))))
-    return f"{dev}|nb{n_b}|p{precision}|L{n_levels}|B{bucket}"
+    return f"{dev}|nb{n_b}|p{precision}|L{n_levels}|B{bucket}|F{FORMS}"
 
 
 def _load() -> dict:
