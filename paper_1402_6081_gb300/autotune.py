@@ -36,7 +36,8 @@ FORMS = 2
 
 # Values per dimension (0 = the library's choice).  interval_kernel: 1 = one
 # CTA per frequency chunk, 3 = paired groups; free_sms: SMs left to levels >= 2
-# beside the persistent products (-1: none); fft_kernel 2: persistent level-0
+# beside the persistent products (-1: none; a plan without these knows one other
+# schedule, whatever the positive value); fft_kernel 2: persistent level-0
 # transforms (FP32, n_b 8 or 16); mac_groups_per_cta: the interaction-list chunk
 DIMENSIONS = {
     "fft_size_interval": {4: [0], 8: [0, 17], 16: [0, 34, 36]},
@@ -137,6 +138,16 @@ def time_options(blocks_list, n_b, levels_list, order, precision, opts, reps=5, 
         lgf_destroy(plan)
 
 
+def runs_persistent(blocks_list, n_b, levels_list, order, precision, opts) -> bool:
+    """Whether a plan with these options has persistent level-0 products."""
+    from . import lgf_destroy, lgf_plan_create_multi, lgf_plan_get_stats
+    plan = lgf_plan_create_multi(blocks_list, n_b, levels_list, order, precision, **opts)
+    try:
+        return lgf_plan_get_stats(plan)["persistent_ctas"] > 0
+    finally:
+        lgf_destroy(plan)
+
+
 def tune_multi(blocks_list, n_b: int, levels_list, order: int, precision: int = LGF_FP32,
                use_cache: bool = True, reps: int = 10) -> dict:
     """Fastest option set for a set of problems solved as one plan (the cache
@@ -164,6 +175,8 @@ def tune_multi(blocks_list, n_b: int, levels_list, order: int, precision: int = 
     if best_ms is None:
         return {}
     for name, values in candidates(n_b, precision):
+        if name == "free_sms" and not runs_persistent(blocks_list, n_b, levels_list, order, precision, best):
+            values = [v for v in values if v >= 0][:2]
         for v in values:
             if v == best.get(name, 0):
                 continue

@@ -25,6 +25,7 @@ def tuner(tmp_path, monkeypatch):
         return 1.0 + len(opts)
 
     monkeypatch.setattr(autotune, "time_options", time_options)
+    monkeypatch.setattr(autotune, "runs_persistent", lambda *a: False, raising=False)
     return lambda: autotune.tune(BLOCKS, 8, 1, 6, lgfm.LGF_FP32), measured, path
 
 
@@ -38,3 +39,11 @@ def test_entries_of_other_forms_are_searched_again(tuner):
     n = len(measured)
     assert tune() == {} and len(measured) == n   # from the cache
     assert set(old) < set(json.loads(path.read_text()))   # the file's other entries stay
+
+
+@pytest.mark.parametrize("persistent,values", [(False, {8}), (True, {-1, 8, 16, 32})])
+def test_free_sms_values_that_build_different_schedules(tuner, monkeypatch, persistent, values):
+    tune, measured, _ = tuner
+    monkeypatch.setattr(autotune, "runs_persistent", lambda *a: persistent, raising=False)
+    tune()
+    assert {o["free_sms"] for o in measured if "free_sms" in o} == values
