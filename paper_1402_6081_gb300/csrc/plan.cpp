@@ -1005,7 +1005,12 @@ static lgf_status build_group(lgf_plan_s* P, const std::vector<HostPlan>& hp, co
     P->grp.aux = daux;
     P->grp.sets = reinterpret_cast<const int4*>(dsets);
     if (f32) {
-        // bands of whole column sets whose images fill about 48 MB of L2
+        // Bands of whole column sets with about 48 MB of images, so that they
+        // stay in L2: equal shares, rounded up to 32 columns, and at least 32
+        // (so 66 MB for the 2112 groups of the 512^3 tori, and 2.1 MB per 128
+        // groups and more from 3000 groups of n_b = 16 on).  The size matters
+        // little beyond: products of the tori 3.97, 3.63 and 3.62 ms for
+        // budgets of 24, 48 and 80 MB.
         const GroupShape gs = group_shape(P->n_b);
         const int64_t column = int64_t(n_groups + 1) * gs.image * int64_t(cplx);
         const int64_t nc = group_columns(P->n_b), most = std::max<int64_t>(32, int64_t(48 << 20) / column);
