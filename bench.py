@@ -143,7 +143,9 @@ def measure_fma_peaks(lgfm, dev: int):
 def profiled_traffic(name: str):
     """DRAM bytes per solve of the dominant phase from its committed ncu
     summary (profiles/<kernel>_torus_box_128_fp32.md), or None when there is
-    none or the kernel sources changed after that capture."""
+    none or the kernel sources changed after that capture.  Every launch is
+    captured alone with cold caches, so the bytes hold reads that the solve
+    finds in L2 (the images that the phase writes and reads back)."""
     import hashlib
     path = os.path.join(ROOT, "profiles", f"{name}_{WORKLOAD}_fp32.md")
     csrc = os.path.join(ROOT, "paper_1402_6081_gb300", "csrc")
@@ -155,7 +157,7 @@ def profiled_traffic(name: str):
                   and " " not in line.split(": ")[0])
         if kv.get("kernel_source_sha256_16") != h:
             return None
-        return int(kv["traffic_bytes_per_launch"])
+        return int(kv["traffic_bytes_per_solve"])
     except Exception:
         return None
 
@@ -784,6 +786,8 @@ def main():
         iso_ms = kt_iso[dom_name][0] / kt_iso[dom_name][1]
         roof = {"bound": "alu", "kernel": dom_name, "achieved": ach, "peak": peak_tf, "unit": "TFLOP/s",
                 "frac": ach / peak_tf, "traffic": profiled_traffic(dom_name),
+                "traffic_how": "DRAM bytes per solve, ncu, every launch alone and cold: an upper bound, images "
+                               "re-read from DRAM that the solve reads from L2",
                 "peak_source": "measured: lgf_measure_fma_peak, best of fma.rn.f32 and fma.rn.f32x2 on all SMs",
                 "peak_derived": derived_tf, "frac_of_derived": ach / derived_tf,
                 "algorithmic": "8 flop x " + work[dom_name][1],

@@ -185,7 +185,8 @@ lgf_status lgf_plan_create(const int32_t *block_ijk, int64_t n_blocks, int32_t n
  *                      length 2 n_b already gives the exact level-1
  *                      convolution; by linearity both levels then share one
  *                      forward FFT, one product pass over the 6^3 blocks of
- *                      the parent neighbourhood (343 kernel offsets) and one
+ *                      the parent neighbourhood (343 kernel offsets; by whole
+ *                      sibling groups 27) and one
  *                      inverse FFT.  1: separate level-1 transforms of length
  *                      S_I, as the level interactions of Sec. 3.1 are listed.
  *   free_sms           schedule of the levels >= 2 beside the level-0 products.
@@ -223,7 +224,10 @@ lgf_status lgf_plan_create(const int32_t *block_ijk, int64_t n_blocks, int32_t n
  *                      kernel vector is centred on index 0, so no twiddle is
  *                      needed), 4.3x fewer rows than the 172-row half table;
  *                      the products gather each offset's coefficients from
- *                      its representative.  0 / 2: the half tables.
+ *                      its representative.  0 / 2: the half tables.  Levels
+ *                      0 and 1 by whole sibling groups have no such table
+ *                      (theirs is 14 of 27 rows): there the option acts on
+ *                      levels >= 2 only, as does the next one.
  *   mac_groups_per_cta the interaction-list chunk of the one-CTA-per-chunk
  *                      products: sibling groups (each with its list of
  *                      neighbour groups) a CTA takes for one frequency chunk,

@@ -21,12 +21,13 @@ namespace lgf {
 // Columns kx S + ky of a group's spectrum; a column is one z line.
 inline int64_t group_columns(int n_b) { return int64_t(4 * n_b) * (2 * n_b + 1); }
 // Stored rows of the kernel table: offsets id 13 .. 26 of 27 (x fastest), row
-// id - 13; offset 26 - id is the conjugate.  A row holds column (ky * NX + kx)
-// by column, kz fastest.
+// id - 13; offset 26 - id is the conjugate.  FP64 [row][column][kz]; FP32
+// [column][row][pair of frequencies] (re, re, im, im), a line's pairs in the
+// order of its image.
 constexpr int kGroupRows = 14;
 
 // FP32 transforms the z lines a band of columns at a time, as part of the
-// products, into images that stay in L2; FP64 keeps all spectra in device
+// products, into images sized to stay in L2; FP64 keeps all spectra in device
 // memory: there the arithmetic, not the traffic, is the bound.
 template <typename T>
 constexpr bool group_banded() { return sizeof(T) == 4; }

@@ -296,8 +296,8 @@ __global__ void __launch_bounds__(256) k_gz_fwd(const cx<double>* xy, const cx<d
 // ---------------------------------------------------------------------------
 // Products and inverse z lines, FP64: bound by the FP64 pipe (1.06 TFLOP/s;
 // 128^3: 1.20 ms, 0.54 G multiply-adds in the products alone take 1.0; the
-// blocks' own products 8.0 ms).  A thread holds one frequency: the 27 kernel
-// values in registers, and per set of 2^3 target groups its 4^3 source groups,
+// blocks' own products 8.0 ms).  A thread holds one frequency: the 14 stored
+// kernel values in registers, and per set of 2^3 target groups its 4^3 source groups,
 // each loaded once and used by every target within reach (216 products).
 // acc += F K, or F conj(K)
 template <bool CONJ>

@@ -1422,7 +1422,6 @@ static lgf_status solve_impl(lgf_plan_s* P, const T* f, T* u, cudaStream_t st) {
     const bool split = Lm >= 2 && uses_persist(P, 0) && P->free_sms < 0;
     auto record = [&](int k, cudaStream_t s) { return conc ? cudaEventRecord(P->join[k], s) : cudaSuccess; };
     auto wait = [&](cudaStream_t s, int k) { return conc ? cudaStreamWaitEvent(s, P->join[k], 0) : cudaSuccess; };
-    // level-0 inverse FFT into u, plus the level-1 field add when given
     // The grouped phases follow one another on st with nothing in between
     // (events do when launches are timed).  Beside the long levels >= 2 chain
     // of the run-time-size kernels, CTAs that started early and wait hold SMs
@@ -1433,6 +1432,7 @@ static lgf_status solve_impl(lgf_plan_s* P, const T* f, T* u, cudaStream_t st) {
     // starts there.
     const bool own = lev[0].n_groups > 0;
     const int chain = P->ev.empty() && !own && !(gen && Lm >= 2) ? 1 : 0;
+    // level-0 inverse FFT into u, plus the level-1 field add when given
     auto c2r0 = [&](const T* add) -> cudaError_t {
         if (P->grouped) {
             const cudaError_t r = Group<T>::inverse(nb, P->grp, group_banded<T>() ? P->gspec : P->gxy, u, add, nI, n3,
@@ -1810,12 +1810,14 @@ static lgf_status create_plan(const int32_t* block_ijk, const int64_t* offsets, 
         }
     }
     if (P->free_sms == 0) {
-        // Default schedule of the persistent products: when levels >= 2 carry
+        // Default schedule of the persistent level-0 products (interval_kernel
+        // 4, 5, and scattered blocks; the grouped form has none): when levels >= 2 carry
         // 7% or more of the level-0/1 pair work they get every SM after the
         // products (split); below that they run beside them on 24 SMs.
         // Measured on GB300 (ms, split / 24 SMs): 128^3 torus (ratio 0.05)
         // 0.280 / 0.252; 256^3 box (0.09) 2.254 / 2.307; 512^3 box (0.11)
-        // 19.82 / 20.43; 512^3 irregular (0.12) 5.48 / 5.85.
+        // 19.82 / 20.43; 512^3 irregular (0.12) 5.48 / 5.85 (when these domains
+        // ran persistent products by default; interval_kernel = 5 today).
         double main = 0, side = 0;
         for (const HostPlan& H : hp) {
             main += double(H.pairs[0] + (H.L >= 1 ? H.pairs[1] : 0)) * double(nw_of(P->S0));
@@ -1829,8 +1831,9 @@ static lgf_status create_plan(const int32_t* block_ijk, const int64_t* offsets, 
         const bool cube_ok = P->prec == LGF_FP32 && cube_fft_supported(P->S0, n_b);
         if (P->fft_kernel == 2 && !cube_ok)
             return fail(LGF_ERR_INVALID_ARG, "lgf_plan_create: fft_kernel 2 needs an FP32 plan with n_b 8 or 16");
-        // default: the per-block form (measured on GB300, 128^3 torus: 28.4 /
-        // 26.7 us forward / inverse in the step against 29.0 / 31.0 us)
+        // default of plans with blocks in their own form: one CTA per block
+        // (measured on GB300, 128^3 torus in that form: 28.4 / 26.7 us forward /
+        // inverse in the step against 29.0 / 31.0 us)
         if (P->fft_kernel == 0) P->fft_kernel = 1;
         if (P->fft_kernel == 2) {
             int n_sm = 0;
@@ -1844,7 +1847,8 @@ static lgf_status create_plan(const int32_t* block_ijk, const int64_t* offsets, 
     }
     // In the split schedule the levels >= 2 chain (aux[1]) runs beside the
     // level-0 FFTs, which fill every SM: at the highest stream priority its
-    // few CTAs go first (measured: 512^3 irregular 5.13e9 -> 5.25e9 points/s).
+    // few CTAs go first (measured in that form: 512^3 irregular 5.13e9 -> 5.25e9
+    // points/s).
     // Beside the persistent products it keeps the default priority (there a
     // head start costs the level-0 forward FFT more than it gains).
     int prio_low = 0, prio_high = 0;
@@ -1852,8 +1856,8 @@ static lgf_status create_plan(const int32_t* block_ijk, const int64_t* offsets, 
     LGF_CUDA(cudaStreamCreateWithFlags(&P->aux[0], cudaStreamNonBlocking));
     const bool split = P->free_sms < 0 && uses_persist(P.get(), 0);
     // Beside the grouped phases it goes first as well (128^3 153 us, 165 at the
-    // default priority; 96^3 ball of 12^3 blocks, FP64, 1351 / 1526), unless the caller asks
-    // the plan to leave room to other work.
+    // default priority; 96^3 ball of 12^3 blocks, FP64, 1351 / 1526), unless the
+    // caller asks the plan to leave room to other work.
     const bool first = split || (P->grouped && !(opts && opts->free_sms > 0));
     LGF_CUDA(cudaStreamCreateWithPriority(&P->aux[1], cudaStreamNonBlocking, first ? prio_high : prio_low));
     LGF_CUDA(cudaEventCreateWithFlags(&P->fork, cudaEventDisableTiming));

@@ -292,8 +292,10 @@ class GpuServer:
     at most fold_points points) run as one multi-problem plan of key (shape,
     k).  k is limited so that the folded plan picks the same product-kernel
     form at every level as the plan of one request (the persistent form is
-    chosen per level by its number of sibling groups, 48 or more), so every
-    folded result has the bits of the same request solved alone.
+    chosen per level by its number of sibling groups, 48 or more; levels 0 and
+    1 count too, although a dense shape's run by whole sibling groups whatever
+    their number), so every folded result has the bits of the same request
+    solved alone.
 
     Large requests (more than big_points points) run on a stream of the
     default priority, the others on high-priority streams, and large plans
