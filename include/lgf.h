@@ -155,7 +155,8 @@ lgf_status lgf_plan_create(const int32_t *block_ijk, int64_t n_blocks, int32_t n
  *                      frequency instead of 8 x 27; scattered blocks, whose
  *                      groups would be mostly padding, keep their own
  *                      transforms: in FP64 problem by problem, in FP32 plan by
- *                      plan; levels >= 1, and that merged pass: 5 for FP32
+ *                      plan (products 5 in FP32 from 48 sibling groups on, else
+ *                      1); levels >= 1: 5 for FP32
  *                      plans where a level has >= 48 sibling groups, elsewhere
  *                      one CTA per (frequency chunk, group range) with the
  *                      packed FP32 products of form 5, 8 warps).  Any other
