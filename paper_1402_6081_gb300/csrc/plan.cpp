@@ -902,8 +902,9 @@ static lgf_status build_host(const int32_t* ijk, int64_t NB, int L, HostPlan& H)
 // group whole, however few of its blocks are there, and takes a set of 2^3
 // target groups at a time, however few of those: where blocks are scattered
 // the blocks' own transforms of 2 n_b are less work.  Counted per problem and
-// summed: sets beyond the first (one set is bound by latency in either form),
-// groups, pairs of neighbouring groups, the blocks those pairs read (where
+// summed: sets beyond the first (one set alone is bound by latency, which
+// favours the groups, except in FP32 at n_b = 16, where a lone group takes 25 us
+// either way and six folded 43 by groups, 27 by their blocks), groups, pairs of neighbouring groups, the blocks those pairs read (where
 // products skip absent sources), blocks.  The weights fit the difference of
 // both forms' solve times over 27 block lists per n_b and precision (boxes,
 // balls, shells, sheets, lines, isolated groups, random blocks and groups, 60 to
@@ -928,7 +929,7 @@ static bool grouping_pays(int prec, int n_b, const HostPlan* hp, size_t n) {
                 ++pairs;
                 sources += members[size_t(g)];
             }
-        sets += int64_t(s.size()) - 1;
+        sets += int64_t(s.size()) - (prec == LGF_FP32 && n_b == 16 ? 0 : 1);
         groups += T.n_groups;
         blocks += H.n_blocks;
     }

@@ -80,3 +80,18 @@ def test_folded_copies_keep_the_form_of_one():
         out = u.cpu().numpy().reshape(3, *f.shape)
         lgfm.lgf_destroy(plan)
         assert all(np.array_equal(o, one) for o in out)
+
+
+@pytest.mark.parametrize("n_b,prec,kernels", [(16, lgfm.LGF_FP32, 3), (16, lgfm.LGF_FP64, 4), (8, lgfm.LGF_FP32, 4)])
+@pytest.mark.parametrize("copies", [1, 6])
+def test_lone_groups(n_b, prec, kernels, copies):
+    # three kernels: the blocks' own form; four: by groups.  Folded copies as alone.
+    blocks = W.full_box_blocks(2)
+    plan = lgfm.lgf_plan_create_multi([blocks] * copies, n_b, [1] * copies, 6, prec)
+    dt = torch.float64 if prec == lgfm.LGF_FP64 else torch.float32
+    f = torch.ones((8 * copies, n_b, n_b, n_b), dtype=dt, device="cuda")
+    lgfm.lgf_solve(plan, f, torch.empty_like(f))
+    lgfm.lgf_plan_sync(plan)
+    n = lgfm.lgf_plan_kernel_launches(plan)
+    lgfm.lgf_destroy(plan)
+    assert n == kernels
